@@ -23,6 +23,7 @@
 #include <string>
 #include <vector>
 
+#include "edge64.cuh"
 #include "gks2l.h"
 #include "mlp.cuh"
 #include "prep.h"
@@ -457,6 +458,18 @@ __global__ void k_harvest(Dev d, const int *perm, float tol, const float *logit_
   if (logits) logits[c] = logit_dev[j];
 }
 
+// the interface and edge units of a form
+template <typename R> __device__ __forceinline__ R iface_any(const Dev &d, int e, int ell) {
+  if constexpr (sizeof(R) == 8) return iface_unit64(d, e, ell);
+  else return iface_unit<R>(d, e, ell);
+}
+template <typename R, bool FUSED = false, bool PAIRED = false, bool POS = false>
+__device__ __forceinline__ bool edge_any(const Dev &d, const Par &p, int e, int ell, int q, int stage, R out[12],
+                                         R *blend = nullptr, R *own = nullptr) {
+  if constexpr (sizeof(R) == 8) return edge_unit64<FUSED, PAIRED, POS>(d, p, e, ell, q, out, blend, own);
+  else return edge_unit<R, FUSED, PAIRED, POS>(d, p, e, ell, q, stage, out, blend, own);
+}
+
 // Each side's own level of layer ell, the mean over the edge's two points:
 // the q = 0 thread writes the L side's, the q = 1 thread the R side's.
 template <typename R>
@@ -493,7 +506,7 @@ __device__ __forceinline__ void iface_body(const Dev &d) {
   int tid = blockIdx.x * blockDim.x + threadIdx.x;
   int e = tid >> 1, ell = tid & 1;
   if (e >= d.ne || !(d.dt[d.inst[d.eL[e]]] > 0)) return;
-  ((R *)d.hc)[ell * d.ne + e] = iface_unit<R>(d, e, ell);
+  ((R *)d.hc)[ell * d.ne + e] = iface_any<R>(d, e, ell);
 }
 
 template <typename R, bool POS = false>
@@ -505,7 +518,7 @@ __device__ __forceinline__ void edge_body(const Dev &d, const Par &p, int stage)
   // its instance's dt is known, so the unit's loads issue at once; only
   // edges of instances still running are written
   R out[12], own[2];
-  edge_unit<R, false, true, POS>(d, p, ee, ell, q, stage, out, nullptr, own);
+  edge_any<R, false, true, POS>(d, p, ee, ell, q, stage, out, nullptr, own);
   const bool ok = e < d.ne && d.dt[d.inst[d.eL[ee]]] > 0;
   own_write<R>(d, e, ell, q, own, ok);
   // the Gauss point q = 0 thread averages the fluxes (out[0..5]), the q = 1
@@ -531,7 +544,7 @@ __device__ __forceinline__ void edge_fused_body(const Dev &d, const Par &p, int 
   int e = tid >> 2, ell = (tid >> 1) & 1, q = tid & 1;
   const int ee = e < d.ne ? e : d.ne - 1;
   R out[12], bl = 0, own[2];
-  const bool done = edge_unit<R, true, true>(d, p, ee, ell, q, stage, out, &bl, own);
+  const bool done = edge_any<R, true, true>(d, p, ee, ell, q, stage, out, &bl, own);
   if (!done) {
     for (int k = 0; k < 12; k++) out[k] = 0;
   }
@@ -578,7 +591,7 @@ __global__ void __launch_bounds__(128) k_edge_deferred(Dev d, Par p, int stage) 
     const int item = d.wl[i < n ? i : n - 1];
     const int e = item >> 1, ell = item & 1;
     R out[12];
-    edge_unit<R>(d, p, e, ell, q, stage, out);
+    edge_any<R>(d, p, e, ell, q, stage, out);
     R avg[6];
 #pragma unroll
     for (int k = 0; k < 6; k++) {
@@ -668,10 +681,10 @@ template <typename R, int BS>
 __global__ void __launch_bounds__(BS) k_iface(Dev d) { iface_body<R>(d); }
 template <typename R, int BS>
 __global__ void __launch_bounds__(BS) k_edge(Dev d, Par p, int stage) { edge_body<R>(d, p, stage); }
-// (the fused kernel's default shapes are held to 768 resident threads per SM,
-// the 80 registers its body compiles to when left alone)
+// (the fused kernel's default shapes are held in FP32 to 768 resident threads
+// per SM, the 80 registers its body compiles to when left alone)
 template <typename R, int BS>
-__global__ void __launch_bounds__(BS, 768 / BS) k_edgef(Dev d, Par p, int stage) { edge_fused_body<R>(d, p, stage); }
+__global__ void __launch_bounds__(BS, sizeof(R) == 4 ? 768 / BS : 1) k_edgef(Dev d, Par p, int stage) { edge_fused_body<R>(d, p, stage); }
 template <typename R, int BS>
 __global__ void __launch_bounds__(BS) k_update(Dev d, Par p, int stage) { update_body<R>(d, p, stage); }
 // the edge solution with the positivity option (one launch shape)
@@ -793,6 +806,7 @@ __global__ void k_step_begin(Dev d, Par p, const double *tend) {
   }
   d.dt[i] = dt;
   ((R *)d.dtR)[i] = (R)dt;
+  ((R *)d.dtR)[d.ninst + i] = dt > 0 ? (R)(1 / dt) : (R)0;
   d.dtbits[i] = DBL_INF_BITS;
 }
 
@@ -981,7 +995,7 @@ size_t layout(gks2l_ctx *c, char *base) {
   d.ref = k.take<double>(2 * ni);
   d.refR = k.take<char>(rs * 2 * ni);
   d.dt = k.take<double>(ni);
-  d.dtR = k.take<char>(rs * ni);
+  d.dtR = k.take<char>(rs * 2 * ni);
   d.t = k.take<double>(ni);
   d.dtbits = k.take<unsigned long long>(ni);
   d.mass = k.take<double>(2 * ni);
@@ -1092,6 +1106,9 @@ Par make_par(const gks2l_ctx *c) {
   p.gam_hi = c->par.weno_gamma_hi; p.weno_eps = c->par.weno_eps;
   p.gf = (float)p.g; p.chif = (float)p.chi; p.epsf = (float)p.eps; p.eps_numf = (float)p.eps_num;
   p.gam_hif = (float)p.gam_hi;
+  p.ig2 = 2 / p.g;
+  p.rg = 1 / std::sqrt(p.g);
+  p.cphi = std::sqrt(p.g / (4 * M_PI));
   p.use_gate = (c->par.indicator == GKS2L_INDICATOR_MLP && c->has_mlp) ? 1 : 0;
   p.harvest = 0;
   p.logit_out = nullptr;

@@ -104,7 +104,7 @@ struct Dev {
   double *ref;              // [inst*2]: R2, R1
   void *refR;               // the same, type R
   double *dt, *t;
-  void *dtR;                // dt, type R
+  void *dtR;                // [2][inst] dt and 1/dt (0 for a stopped instance), type R
   unsigned long long *dtbits;
   double *mass;             // [inst*2 + layer]
   int *status;
@@ -115,6 +115,7 @@ struct Dev {
 struct Par {
   double g, chi, cfl, eps, eps_num, gam_hi, weno_eps;
   float gf, chif, epsf, eps_numf, gam_hif;   // the same in single precision
+  double ig2, rg, cphi;                      // 2/G, 1/sqrt(G), sqrt(G/(4 pi)): the double form's edge solution
   int use_gate;                              // learned gate active
   float *logit_out;                          // gate logits per cell (device order), or null
   int all_active;                            // reconstruct every instance (harvesting)
@@ -174,6 +175,13 @@ template <> __host__ __device__ __forceinline__ float r_expm1<float>(float x) { 
 template <typename R> __host__ __device__ __forceinline__ R r_sqrt(R x);
 template <> __host__ __device__ __forceinline__ double r_sqrt<double>(double x) { return sqrt(x); }
 template <> __host__ __device__ __forceinline__ float r_sqrt<float>(float x) { return sqrtf(x); }
+__host__ __device__ __forceinline__ double r_rsqrt(double x) {
+#ifdef __CUDA_ARCH__
+  return rsqrt(x);
+#else
+  return 1 / sqrt(x);
+#endif
+}
 template <typename R> __host__ __device__ __forceinline__ R r_abs(R x) { return x < 0 ? -x : x; }
 
 // the bits of a double as a signed integer (> 0: positive, nonzero, and
@@ -299,6 +307,23 @@ __host__ __device__ inline void recon_p3(const CellOps<R> &o, const R rhs[NCOL],
   }
 }
 
+// t / a and t / b from one reciprocal (in FP64 5 pipe slots against 8 for each
+// division), or by division where the product a b leaves the normal range
+template <typename R>
+__host__ __device__ __forceinline__ void ratios2(R t, R a, R b, R r[2]) {
+  const R ab = a * b;
+  // 2^-960 <= ab < 2^960 by the exponent's bits (off the FP64 pipe)
+  const int ex = (int)((dbits((double)ab) >> 52) & 0x7ff);
+  if (ex > 63 && ex < 1983) {
+    const R i = t * ((R)1 / ab);
+    r[0] = i * b;
+    r[1] = i * a;
+  } else {
+    r[0] = t / a;
+    r[1] = t / b;
+  }
+}
+
 // The result goes to the cell's side records: straight to global memory, or,
 // with `stage` set, to a block's staging tile [layer][cell in tile][NREC]
 // (o.stride cells per layer) that the block then writes out with 16-byte
@@ -323,8 +348,18 @@ __host__ __device__ inline void recon_finish(const Dev &d, const Par &p, const C
     }
     R bh = 0;
     int idx = 0;
-    for (int k = 0; k < 9; k++)
-      for (int l = k; l < 9; l++) bh += o.bq[(idx++) * S + I] * a[k] * a[l];
+    for (int k = 0; k < 9; k++) {
+      if (sizeof(R) == 8) {
+        // a_k times the row's sum: 54 operations in place of 90 (with the
+        // weights' shared reciprocals k_recon<double> goes from 404 to 344 FP64
+        // operations per cell and variable, 2224 -> 1897 us at 501 k triangles)
+        R row = 0;
+        for (int l = k; l < 9; l++) row += o.bq[(idx++) * S + I] * a[l];
+        bh += a[k] * row;
+      } else {
+        for (int l = k; l < 9; l++) bh += o.bq[(idx++) * S + I] * a[k] * a[l];
+      }
+    }
     beta[0] = bh;
     R tz = (r_abs<R>(bh - beta[1]) + r_abs<R>(bh - beta[2]) + r_abs<R>(bh - beta[3])) * (R)(1.0 / 3.0);
     // the variable's value (reference + deviation) scales the regulariser
@@ -333,16 +368,31 @@ __host__ __device__ inline void recon_finish(const Dev &d, const Par &p, const C
     if (v == 0) Q0 += refR[2 * d.inst[j]];
     if (v == 3) Q0 += refR[2 * d.inst[j] + 1];
     R eps = ((const R *)d.epsA)[j] * (1 + Q0 * Q0);
-    R w[4], ws = 0;
     const R gam[4] = {gh, gl, gl, gl};
-    for (int k = 0; k < 4; k++) {
-      R r = tz / (beta[k] + eps);
-      w[k] = gam[k] * (1 + r * r);
-      ws += w[k];
+    if (sizeof(R) == 8) {
+      R u[4], ws = 0;
+      for (int k = 0; k < 4; k += 2) {
+        R r[2];
+        ratios2<R>(tz, beta[k] + eps, beta[k + 1] + eps, r);
+        for (int i = 0; i < 2; i++) {
+          u[k + i] = 1 + r[i] * r[i];
+          ws += gam[k + i] * u[k + i];
+        }
+      }
+      const R iw = 1 / ws;
+      fac = u[0] * iw;
+      for (int f = 0; f < 3; f++) wf[f] = u[1 + f] * (gl * iw);
+    } else {
+      R w[4], ws = 0;
+      for (int k = 0; k < 4; k++) {
+        R r = tz / (beta[k] + eps);
+        w[k] = gam[k] * (1 + r * r);
+        ws += w[k];
+      }
+      R iw = 1 / ws;
+      fac = w[0] * iw / gh;
+      for (int f = 0; f < 3; f++) wf[f] = w[1 + f] * iw;
     }
-    R iw = 1 / ws;
-    fac = w[0] * iw / gh;
-    for (int f = 0; f < 3; f++) wf[f] = w[1 + f] * iw;
     if (p.harvest) {
       R dv = r_abs<R>(fac - 1);
       for (int f = 0; f < 3; f++) {
