@@ -110,7 +110,7 @@ __host__ __device__ __forceinline__ double blend64(double dl, double ul, double 
 // iface_unit in the double form
 __host__ __device__ inline double iface_unit64(const Dev &d, int e, int ell) {
   using O = D64;
-  const int NE = d.ne, N = d.cs;
+  const int NE = d.ne;
   const double *en = (const double *)d.en;
   const double n0 = en[e], n1 = en[NE + e];
   double lev[2][2], un[2][2];
@@ -118,7 +118,7 @@ __host__ __device__ inline double iface_unit64(const Dev &d, int e, int ell) {
     const double *xs = sd == 0 ? (const double *)d.exiL : (const double *)d.exiR;
     double fr[4], w[NREC];
     face_frame(d, n0, n1, sd == 0 ? 0 : d.exf[e], fr);
-    load_rec<double, NREC>((const double *)d.srec + ((size_t)ell * N + (sd == 0 ? d.eL[e] : d.eR[e])) * NREC, w);
+    load_rec<double, NREC>(d, ell, sd == 0 ? d.eL[e] : d.eR[e], w);
     for (int q = 0; q < 2; q++) {
       double m[10];
       monos64(xs[(2 * q) * NE + e], xs[(2 * q + 1) * NE + e], m);
@@ -160,9 +160,8 @@ template <bool OTHER>
 __host__ __device__ __forceinline__ void side64(const Dev &d, int ell, int c, int xf, const double fr[4],
                                                 const double m[10], double href, Side64 &s) {
   using O = D64;
-  const int N = d.cs;
   double w[NREC];
-  load_rec<double, NREC>((const double *)d.srec + ((size_t)ell * N + c) * NREC, w);
+  load_rec<double, NREC>(d, ell, c, w);
   const double ih = w[11];
   double fs[4] = {O::mul(fr[0], ih), O::mul(fr[1], ih), 0, 0};
   fs[2] = -fs[1];
@@ -200,7 +199,7 @@ __host__ __device__ __forceinline__ void side64(const Dev &d, int ell, int c, in
   s.oth[0] = s.oth[1] = 0;
   if (OTHER) {
     double wo[12];
-    load_rec<double, 12>((const double *)d.srec + ((size_t)(1 - ell) * N + c) * NREC, wo);
+    load_rec<double, 12>(d, 1 - ell, c, wo);
     level_dirs(wo, m, fs, s.oth);
   }
 }
@@ -492,14 +491,15 @@ __host__ __device__ inline bool edge_unit64(const Dev &d, const Par &p, int e, i
       D[sd][k] = O::fma(cf, FUSED ? s[sd].oth[k] : O::fma(w, s[sd].oth[k], O::mul(w1, pl[sd][k])), s[sd].lev[k]);
   if (FUSED) *blend = blend64(s[0].d, s[0].U, s[1].d, s[1].U);
   if (POS) {
-    const int N = d.cs, vm = ell == 0 ? 4 : 1;
+    const int N = d.cs;
     const bool fl[2] = {d.pos_flag[ell * N + cL] != 0, d.pos_flag[ell * N + cR] != 0};
     if (fl[0] || fl[1]) {
-      const double *hb = (const double *)d.pos_hbar, *dq = (const double *)d.dq;
+      const double *hb = (const double *)d.pos_hbar;
       double un[2], ut[2];
       for (int sd = 0; sd < 2; sd++) {
         const int c = sd == 0 ? cL : cR;
-        const double mx = dq[vm * N + c], my = dq[(vm + 1) * N + c], ihb = 1 / hb[ell * N + c];
+        const double *mq = dq_at<double>(d, ell == 0 ? 2 : 1, c);
+        const double mx = mq[0], my = mq[1], ihb = 1 / hb[ell * N + c];
         un[sd] = O::mul(O::fma(mx, fr[sd][0], O::mul(my, fr[sd][1])), ihb);
         ut[sd] = O::mul(O::fma(mx, fr[sd][2], O::mul(my, fr[sd][3])), ihb);
       }

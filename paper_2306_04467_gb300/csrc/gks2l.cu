@@ -2,9 +2,10 @@
 //
 // One S2O4 stage (arXiv 2306.04467, Eq. SWE-fully-discrete) over
 // structure-of-arrays data in a Morton-renumbered cell order:
-//   k_recon   (32 cells x 6 variables per block) compact P3/WENO reconstruction
-//             (Sec. 3.4); the tile's operator rows arrive in shared memory by
-//             bulk copy (cp.async.bulk) behind an mbarrier
+//   k_recon   (32 cells x 6 variables per block, two per thread in FP32)
+//             compact P3/WENO reconstruction (Sec. 3.4); the tile's operator
+//             rows arrive in shared memory by bulk copy (cp.async.bulk)
+//             behind mbarriers
 //   k_iface   (edge x layer)         blended interface levels h-hat (Sec. 2.3)
 //   k_edge    (edge x layer x point) gas-kinetic interface solution (Eq. SWE-2nd-order)
 //   k_update  (cell)                 fluxes, sources, S2O4 update, Gauss-theorem
@@ -45,30 +46,27 @@ constexpr int GATE_LD = 40;             // padded row stride of the gate feature
 // ---------------------------------------------------------------- TMA staging
 // The reconstruction's operator rows of one tile of TW cells, [row][TW] per
 // group, stored contiguously per tile in global memory and copied as they lie
-// into shared memory by the bulk-copy engine. The groups come in the order
-// the copies need them: what every tile uses (P3 least-squares rows, monomial
-// means, stencil cells and their transforms), then what only tiles with a
-// troubled cell use (P1 candidate rows, smoothness forms), so a tile the gate
-// calls smooth fetches one prefix.
+// into shared memory by the bulk-copy engine, in two copies: what every tile
+// uses (P3 least-squares rows, monomial means), then what only tiles with a
+// troubled cell use (P1 candidate rows, smoothness forms). In FP32 both are
+// asked for at once and the second arrives while the P3 fit runs; in FP64,
+// where shared memory for both would leave three blocks per SM (measured 287
+// against 269 us at 65,522 triangles), the second follows the fit into the
+// space of the LSQ rows.
 template <typename R> struct TileLayout {
   static constexpr unsigned LSQ = 0;
   static constexpr unsigned MM = LSQ + kCoef * kCols * TW * sizeof(R);
-  static constexpr unsigned ST = MM + 7 * TW * sizeof(R);
-  static constexpr unsigned SX = ST + kSlots * TW * 4;
-  static constexpr unsigned P1 = SX + kSlots * TW;
+  static constexpr unsigned P1 = MM + 7 * TW * sizeof(R);
   static constexpr unsigned BQ = P1 + 30 * TW * sizeof(R);
   static constexpr unsigned END = BQ + kBeta * TW * sizeof(R);
-  static constexpr unsigned TILE = (END + 127) / 128 * 128;   // tile stride in global memory
+  static constexpr unsigned TILE = END;                        // tile stride in global memory
   static constexpr unsigned TX_LINEAR = P1;                    // bytes of the first copy
   static constexpr unsigned TX2 = END - P1;                    // bytes of the second copy
-  // Shared memory holds the first copy; a tile with a troubled cell fetches
-  // the second after the P3 fit, into the space of the LSQ rows, which the
-  // side-record staging then follows.
-  static constexpr unsigned LATE = LSQ;
-  static constexpr unsigned STG = LATE + (TX2 + 127) / 128 * 128;
-  static constexpr unsigned BAR = (P1 + 127) / 128 * 128;      // the mbarrier, after the first copy
-  static_assert(STG + 2 * TW * NREC * sizeof(R) <= MM, "late rows and side-record staging fit in the LSQ rows");
-  static_assert(P1 % 16 == 0 && END % 16 == 0, "bulk copies move multiples of 16 bytes");
+  static constexpr bool REUSE = sizeof(R) == 8;                // the second copy takes the LSQ rows' space
+  static constexpr unsigned LATE = REUSE ? LSQ : P1;           // where the second copy lands
+  static constexpr unsigned BAR = REUSE ? P1 : END;            // two mbarriers
+  static_assert(2 * TW * NREC * sizeof(R) <= MM && TX2 <= MM, "the staged side records and the second copy fit there");
+  static_assert(P1 % 128 == 0 && END % 128 == 0, "bulk copies move whole lines");
 };
 
 __device__ __forceinline__ unsigned smem_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
@@ -112,13 +110,24 @@ __device__ __forceinline__ bool mbar_wait_bounded(void *bar, unsigned parity, un
 }
 
 // ------------------------------------------------------------------ kernels
-// resident reconstruction blocks per SM the register budget is held to (in
-// FP32 eight, as many as the registers allow: a block per tile keeps 48
-// warps per SM on the neighbour gathers; persistent blocks with two operator
-// buffers, fetching the next tile during the current one, halve the warps
-// and run slower)
-template <typename R> struct ReconOcc { static constexpr int value = 8; };
-template <> struct ReconOcc<double> { static constexpr int value = 4; };
+// The reconstruction's blocks: 32 cells, one warp per pair of variables in
+// FP32 and per variable in FP64. Measured bounds of the FP32 kernel with one
+// variable per thread: the shared-memory and L1 pipe at 75% (each of a tile's
+// 153 operator rows read by six warps, the gathers one value at a time, the
+// records staged with four-way bank conflicts) and the chain copy, stencil,
+// gather, fit, second copy, with DRAM at 49%. Hence two variables per thread
+// (each operator row read by three warps, paired gathers), gathers issued
+// beside the operator copies from the stencil's own array, both copies issued
+// at once, and records written straight from registers: 356 -> 245 us plain
+// and 281 -> 197 us gated at 1.04 M triangles.
+// FP64 is bound by its pipe and keeps the parallelism of one variable per
+// thread. Blocks per SM: what the tiles' shared memory allows.
+template <typename R> struct ReconCfg {
+  static constexpr int VP = 2, BLOCKS = 7;
+};
+template <> struct ReconCfg<double> {
+  static constexpr int VP = 1, BLOCKS = 4;
+};
 template <typename R> constexpr unsigned recon_smem() { return TileLayout<R>::BAR + 16; }
 
 // Positivity option (not in the paper), on a tile's staged side records: for
@@ -162,39 +171,57 @@ __device__ void recon_positivity(const Dev &d, const Par &p, int j, int lay, R *
 }
 
 template <typename R, bool POS = false>
-__global__ void __launch_bounds__(192, ReconOcc<R>::value) k_recon(Dev d, Par p) {
+__global__ void __launch_bounds__(TW * 6 / ReconCfg<R>::VP, ReconCfg<R>::BLOCKS) k_recon(Dev d, Par p) {
   using T = TileLayout<R>;
+  constexpr int VP = ReconCfg<R>::VP;
   extern __shared__ __align__(128) unsigned char sm[];
-  const int j0 = blockIdx.x * TW;
-  void *bar = sm + T::BAR;
+  const int j0 = blockIdx.x * TW, lane = threadIdx.x;
+  void *bar = sm + T::BAR, *bar2 = sm + T::BAR + 8;
   // troubled-cell gate: the previous reconstruction left the mask of this
   // tile's cells it calls smooth; a tile whose cells all take the linear
   // weights needs neither the P1 rows nor the smoothness forms
   const bool gate_on = p.use_gate && !p.harvest;
   const unsigned lin_mask = gate_on ? d.gate_mask[blockIdx.x] : 0u;
   const bool all_linear = lin_mask == 0xffffffffu;
-  const bool lead = threadIdx.x == 0 && threadIdx.y == 0;
-  const unsigned char *src = (const unsigned char *)d.ops + (size_t)blockIdx.x * T::TILE;
-  if (lead) {
+  if (lane == 0 && threadIdx.y == 0) {
+    const unsigned char *src = (const unsigned char *)d.ops + (size_t)blockIdx.x * T::TILE;
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(bar)) : "memory");
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(bar2)) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(T::TX_LINEAR)
                  : "memory");
     bulk_load(sm, src, T::TX_LINEAR, bar);
+    if (!T::REUSE && !all_linear) {
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar2)), "r"(T::TX2)
+                   : "memory");
+      bulk_load(sm + T::LATE, src + T::P1, T::TX2, bar2);
+    }
   }
-  // the cell's activity (a chain of two loads) resolves during the copies
-  const int j = j0 + threadIdx.x, v = threadIdx.y;
-  const bool active = j < d.nt && (p.all_active || d.dt[d.inst[j]] > 0);
+  // the stencil's values and the cell's activity (a chain of two loads)
+  // arrive beside the copies
+  const int j = j0 + lane, jj = min(j, d.nt - 1);
+  const int pair = VP == 2 ? threadIdx.y : pair_of(threadIdx.y), comp = VP == 2 ? 0 : comp_of(threadIdx.y);
+  const bool active = j < d.nt && (p.all_active || running(d, d.inst[jj]));
+  R rhs[VP][NCOL], a[VP][9], q0[VP], rec[VP][12];
+  auto gather = [&] {
+    int st[NSLOT];
+#pragma unroll
+    for (int s = 0; s < NSLOT; s++) st[s] = d.st_cell[(size_t)s * d.cs + jj];
+    recon_gather<R, VP>(d, jj, pair, comp, st, d.tile_xf[blockIdx.x] != 0, rhs, q0);
+  };
+  if (VP == 2) gather();   // (the double form's registers do not hold them across the wait)
   __syncthreads();
   const bool landed =
       mbar_wait_bounded(bar, 0, 1000000000ull, p.staging_polls > 0 ? p.staging_polls - 1 : (1 << 24));
   if (!__syncthreads_and(landed)) {
-    // the copies did not land in time: report, wait for them once more
+    // the copies did not land in time: report, wait for both once more
     // (bounded, a second) so no copy outlives the block, and leave (all
     // threads); if they still have not landed, the block's shared memory may
     // yet be written after it exits, which a second bit records
-    if (lead) atomicOr(d.status, ST_TIMEOUT);
-    if (!landed && !mbar_wait_bounded(bar, 0, 1000000000ull)) atomicOr(d.status, ST_COPY_LOST);
+    if (lane == 0 && threadIdx.y == 0) atomicOr(d.status, ST_TIMEOUT);
+    if (!mbar_wait_bounded(bar, 0, 1000000000ull) ||
+        (!T::REUSE && !all_linear && !mbar_wait_bounded(bar2, 0, 1000000000ull)))
+      atomicOr(d.status, ST_COPY_LOST);
     return;
   }
   CellOps<R> o;
@@ -202,70 +229,68 @@ __global__ void __launch_bounds__(192, ReconOcc<R>::value) k_recon(Dev d, Par p)
   o.p1 = (const R *)(sm + T::LATE);
   o.bq = (const R *)(sm + T::LATE + (T::BQ - T::P1));
   o.mm = (const R *)(sm + T::MM);
-  o.st = (const int *)(sm + T::ST);
-  o.sx = (const int8_t *)(sm + T::SX);
   o.stride = TW;
-  o.idx = threadIdx.x;
-  const bool linear = ((lin_mask >> threadIdx.x) & 1u) != 0;
-  if (gate_on && v == 0) {
+  o.idx = lane;
+  if (VP == 1) gather();
+  const bool linear = ((lin_mask >> lane) & 1u) != 0;
+  if (gate_on && threadIdx.y == 0) {
     const unsigned ns = __popc(__ballot_sync(FULL, active && linear)), nc = __popc(__ballot_sync(FULL, active));
-    if (threadIdx.x == 0) {
+    if (lane == 0) {
       atomicAdd(&d.gate_count[0], (unsigned long long)ns);
       atomicAdd(&d.gate_count[1], (unsigned long long)nc);
     }
   }
-  R rhs[NCOL], a[9];
-  if (active) {
-    recon_gather<R>(d, o, j, v, rhs);
-    recon_p3<R>(o, rhs, a);
-  }
-  // every warp is done with the LSQ rows: their space takes the late rows
-  // (tiles with a troubled cell) and stages the side records
-  __syncthreads();
+  if (active) recon_p3<R, VP>(o, rhs, a);
   if (!all_linear) {
-    if (lead) {
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(T::TX2)
-                   : "memory");
-      bulk_load(sm + T::LATE, src + T::P1, T::TX2, bar);
+    if (T::REUSE) {
+      __syncthreads();   // every warp is done with the LSQ rows
+      if (lane == 0 && threadIdx.y == 0) {
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar2)), "r"(T::TX2)
+                     : "memory");
+        bulk_load(sm + T::LATE, (const unsigned char *)d.ops + (size_t)blockIdx.x * T::TILE + T::P1, T::TX2, bar2);
+      }
     }
-    const bool late = mbar_wait_bounded(bar, 1, 1000000000ull);
-    if (!__syncthreads_and(late)) {
-      if (lead) atomicOr(d.status, ST_TIMEOUT);
-      if (!late && !mbar_wait_bounded(bar, 1, 1000000000ull)) atomicOr(d.status, ST_COPY_LOST);
+    const bool late = mbar_wait_bounded(bar2, 0, 1000000000ull);
+    if (POS ? !__syncthreads_and(late) : !__all_sync(FULL, late)) {
+      if (lane == 0) atomicOr(d.status, ST_TIMEOUT);
+      if (!late && !mbar_wait_bounded(bar2, 0, 1000000000ull)) atomicOr(d.status, ST_COPY_LOST);
       return;
     }
   }
-  R *stg = (R *)(sm + T::STG);
-  if (active) recon_finish<R>(d, p, o, j, v, rhs, a, linear, stg);
-  if (v == 5 && j < d.nt) {
-    // the constant words: 1/h_s and the bottom slope
-    R *r0 = stg + (size_t)threadIdx.x * NREC, *r1 = stg + (size_t)(TW + threadIdx.x) * NREC;
-    const R ih = ((const R *)d.ihsR)[j];
-    r0[11] = ih;
-    r1[11] = ih;
-    r0[23] = ((const R *)d.bgR)[j];
-    r0[35] = ((const R *)d.bgR)[d.cs + j];
-    r1[23] = r1[35] = 0;
+  if (active) recon_finish<R, VP>(d, p, o, jj, pair, comp, rhs, a, q0, linear, rec);
+  constexpr int V = 16 / sizeof(R), NVEC = 12 / V;      // values per vector, vectors per slot
+  uint4 *dst = reinterpret_cast<uint4 *>((R *)d.srec + (size_t)blockIdx.x * (2 * NREC * TW)) + lane;
+  if (!POS) {
+    // a warp's 32 vectors are contiguous
+    if (!active) return;
+    for (int i = 0; i < VP; i++) {
+      int layer;
+      const int slot = slot_of(pair, VP == 2 ? i : comp, layer);
+      for (int k = 0; k < NVEC; k++) {
+        uint4 t;
+        memcpy(&t, rec[i] + k * V, 16);
+        dst[((layer * 3 + slot) * NVEC + k) * TW] = t;
+      }
+    }
+    return;
+  }
+  // positivity: a layer's whole records meet in the space of the LSQ rows
+  R *stg = (R *)(sm + T::LSQ);
+  __syncthreads();
+  if (active) {
+    for (int i = 0; i < VP; i++) {
+      int layer;
+      const int slot = slot_of(pair, VP == 2 ? i : comp, layer);
+      for (int k = 0; k < 12; k++) stg[(layer * TW + lane) * NREC + slot * 12 + k] = rec[i][k];
+    }
   }
   __syncthreads();
-  if (POS) {
-    if (threadIdx.y < 2 && j < d.nt && active) {
-      recon_positivity<R>(d, p, j, threadIdx.y, stg + ((size_t)threadIdx.y * TW + threadIdx.x) * NREC);
-    }
-    __syncthreads();
-  }
-  // coalesced write-out: each layer's records of the tile are contiguous, and
-  // so is the staging tile, so the copy moves 16-byte vectors
-  constexpr int V = 16 / sizeof(R);                 // values per vector
-  constexpr int NV_LAYER = TW * NREC / V;           // vectors per layer
-  const int tid = threadIdx.y * TW + threadIdx.x;
-  const int ncell = min(TW, d.nt - j0);             // the last tile may be partial
-  for (int i = tid; i < 2 * NV_LAYER; i += TW * 6) {
-    const int lay = i / NV_LAYER, r = i - lay * NV_LAYER;
-    if (r * V < ncell * NREC)
-      reinterpret_cast<uint4 *>((R *)d.srec + ((size_t)lay * d.cs + j0) * NREC)[r] =
-          reinterpret_cast<const uint4 *>(stg + lay * TW * NREC)[r];
+  if (threadIdx.y < 2 && active) recon_positivity<R>(d, p, j, threadIdx.y, stg + (threadIdx.y * TW + lane) * NREC);
+  __syncthreads();
+  if (active) {
+    for (int i = threadIdx.y; i < 6 * NVEC; i += 6 / VP)
+      dst[i * TW] = *reinterpret_cast<const uint4 *>(stg + ((i / (3 * NVEC)) * TW + lane) * NREC + (i % (3 * NVEC)) * V);
   }
 }
 
@@ -291,10 +316,10 @@ __global__ void __launch_bounds__(128) k_gate(Dev d, Par p) {
   const int ntile = (d.nt + TW - 1) / TW;
   for (int tile = blockIdx.x * 4 + wid; tile < ntile; tile += gridDim.x * 4) {
     const int j = tile * TW + lane;
-    const bool active = j < d.nt && (p.all_active || d.dt[d.inst[j]] > 0);
+    const bool active = j < d.nt && (p.all_active || running(d, d.inst[j]));
     float f[24];
     if (active) {
-      gate_features<R>(d, j, d.st_cell, d.st_xf, d.cs, j, f);
+      gate_features<R>(d, j, f);
     } else {
       for (int k = 0; k < 24; k++) f[k] = 0.f;
     }
@@ -376,9 +401,9 @@ __global__ void __launch_bounds__(GATE_TC_M) k_gate_tc(Dev d, Par p) {
   bool failed = false;
   for (int tile = blockIdx.x; tile < ntile && !failed; tile += gridDim.x) {
     const int j = tile * GATE_TC_M + tid;
-    const bool active = j < d.nt && (p.all_active || d.dt[d.inst[j]] > 0);
+    const bool active = j < d.nt && (p.all_active || running(d, d.inst[j]));
     float f[32];
-    if (active) gate_features<R>(d, j, d.st_cell, d.st_xf, d.cs, j, f);
+    if (active) gate_features<R>(d, j, f);
     else
       for (int k = 0; k < 24; k++) f[k] = 0.f;
     for (int k = 24; k < 32; k++) f[k] = 0.f;
@@ -450,7 +475,7 @@ __global__ void k_harvest(Dev d, const int *perm, float tol, const float *logit_
   if (j >= d.nt) return;
   const size_t c = (size_t)perm[j];
   float f[24];
-  gate_features<R>(d, j, d.st_cell, d.st_xf, d.cs, j, f);
+  gate_features<R>(d, j, f);
   for (int k = 0; k < 24; k++) X[c * 24 + k] = f[k];
   float dv = 0.f;
   for (int v = 0; v < NV; v++) dv = fmaxf(dv, d.wdev[v * d.cs + j]);
@@ -505,7 +530,7 @@ template <typename R>
 __device__ __forceinline__ void iface_body(const Dev &d) {
   int tid = blockIdx.x * blockDim.x + threadIdx.x;
   int e = tid >> 1, ell = tid & 1;
-  if (e >= d.ne || !(d.dt[d.inst[d.eL[e]]] > 0)) return;
+  if (e >= d.ne || !running(d, d.inst[d.eL[e]])) return;
   ((R *)d.hc)[ell * d.ne + e] = iface_any<R>(d, e, ell);
 }
 
@@ -519,7 +544,7 @@ __device__ __forceinline__ void edge_body(const Dev &d, const Par &p, int stage)
   // edges of instances still running are written
   R out[12], own[2];
   edge_any<R, false, true, POS>(d, p, ee, ell, q, stage, out, nullptr, own);
-  const bool ok = e < d.ne && d.dt[d.inst[d.eL[ee]]] > 0;
+  const bool ok = e < d.ne && running(d, d.inst[d.eL[ee]]);
   own_write<R>(d, e, ell, q, own, ok);
   // the Gauss point q = 0 thread averages the fluxes (out[0..5]), the q = 1
   // thread the interface values (out[6..11]): each sends the other its half
@@ -558,7 +583,7 @@ __device__ __forceinline__ void edge_fused_body(const Dev &d, const Par &p, int 
     const R mine = q == 0 ? out[k] : out[6 + k], theirs = q == 0 ? out[6 + k] : out[k];
     avg[k] = (R)0.5 * (mine + __shfl_xor_sync(FULL, theirs, 1));
   }
-  const bool ok = e < d.ne && d.dt[d.inst[d.eL[ee]]] > 0;
+  const bool ok = e < d.ne && running(d, d.inst[d.eL[ee]]);
   own_write<R>(d, e, ell, q, own, ok);
   // deferred units to the worklist, one atomic per warp
   const bool push = ok && q == 0 && !done;
@@ -817,12 +842,22 @@ __global__ void k_mirrors(Dev d, const int *perm, const double *grad_caller) {
   int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= d.nt) return;
   const int N = d.cs, in = d.inst[j], c = perm[j];
-  R *dq = (R *)d.dq, *dg = (R *)d.dg;
   const double R2 = d.ref[2 * in], R1 = d.ref[2 * in + 1];
-  dq[j] = (R)(d.avg[j] - R2);
-  dq[3 * N + j] = (R)((d.avg[3 * N + j] + d.bmean[j]) - R1);
-  for (int v : {1, 2, 4, 5}) dq[v * N + j] = (R)d.avg[v * N + j];
-  for (int k = 0; k < 12; k++) dg[k * N + j] = (R)(grad_caller ? grad_caller[(size_t)k * d.nt + c] : 0.0);
+  for (int i = 0; i < NPAIR; i++) {
+    const int v0 = var_of(i, 0), v1 = var_of(i, 1);
+    R q[2] = {(R)d.avg[v0 * N + j], (R)d.avg[v1 * N + j]}, g[4] = {0, 0, 0, 0};
+    if (i == 0) {
+      q[0] = (R)(d.avg[j] - R2);
+      q[1] = (R)((d.avg[3 * N + j] + d.bmean[j]) - R1);
+    }
+    if (grad_caller)
+      for (int k = 0; k < 2; k++) {
+        g[k] = (R)grad_caller[(size_t)(2 * v0 + k) * d.nt + c];
+        g[2 + k] = (R)grad_caller[(size_t)(2 * v1 + k) * d.nt + c];
+      }
+    store_n<R, 2>(dq_at<R>(d, i, j), q);
+    store_n<R, 4>(dg_at<R>(d, i, j), g);
+  }
   ((R *)d.hrefc)[j] = (R)(R1 - d.bmean[j]);
 }
 
@@ -841,8 +876,12 @@ __global__ void k_grad_out(Dev d, const int *perm, double *out) {
   int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= d.nt) return;
   const int c = perm[j];
-  const R *dg = (const R *)d.dg;
-  for (int k = 0; k < 12; k++) out[(size_t)k * d.nt + c] = (double)dg[k * d.cs + j];
+  for (int i = 0; i < NPAIR; i++) {
+    R g[4];
+    load_n<R, 4>(dg_at<R>(d, i, j), g);
+    for (int m = 0; m < 2; m++)
+      for (int k = 0; k < 2; k++) out[(size_t)(2 * var_of(i, m) + k) * d.nt + c] = (double)g[2 * m + k];
+  }
 }
 
 // caller order (stride nt) <-> device order (stride cs)
@@ -951,6 +990,7 @@ size_t layout(gks2l_ctx *c, char *base) {
   d.bgy = k.take<double>(nt);
   d.st_cell = k.take<int>(kSlots * cs);
   d.st_xf = k.take<int8_t>(kSlots * cs);
+  d.tile_xf = k.take<int>(cs / TW);
   d.ops = k.take<char>((cs / TW) * (rs == 4 ? TileLayout<float>::TILE : TileLayout<double>::TILE));
   d.plane = k.take<char>(rs * 6 * cs);
   d.cedge = k.take<int>(3 * cs);
@@ -1061,17 +1101,11 @@ int upload_tiles(gks2l_ctx *c) {
     for (size_t t = 0; t < nb; t++) {
       unsigned char *b = buf.data() + t * T::TILE;
       R *lsq = (R *)(b + T::LSQ), *mm = (R *)(b + T::MM), *p1 = (R *)(b + T::P1), *bq = (R *)(b + T::BQ);
-      int *st = (int *)(b + T::ST);
-      int8_t *sx = (int8_t *)(b + T::SX);
       for (int i = 0; i < TW; i++) {
         const size_t j = (t0 + t) * TW + i;
         if (j >= nt) break;
         for (int r = 0; r < kCoef * kCols; r++) lsq[r * TW + i] = (R)P.lsq[r * nt + j];
         for (int r = 0; r < 7; r++) mm[r * TW + i] = (R)P.mmean[r * nt + j];
-        for (int r = 0; r < kSlots; r++) {
-          st[r * TW + i] = P.st_cell[r * nt + j];
-          sx[r * TW + i] = P.st_xf[r * nt + j];
-        }
         for (int r = 0; r < 30; r++) p1[r * TW + i] = (R)P.p1op[r * nt + j];
         for (int r = 0; r < kBeta; r++) bq[r * TW + i] = (R)P.bq[r * nt + j];
       }
@@ -1089,12 +1123,14 @@ int upload_bathymetry(gks2l_ctx *c) {
   std::vector<double> bm, bx, by, e0, e1;
   bathymetry(c->prep, c->has_b ? c->bvert.data() : nullptr, bm, bx, by, e0, e1);
   std::vector<double> bg(2 * (size_t)c->prep.nt);
-  std::copy(bx.begin(), bx.end(), bg.begin());
-  std::copy(by.begin(), by.end(), bg.begin() + c->prep.nt);
+  for (size_t j = 0; j < bx.size(); j++) {
+    bg[2 * j] = bx[j];
+    bg[2 * j + 1] = by[j];
+  }
   int rc;
   if ((rc = upload(c, c->d.bmean, bm)) || (rc = upload(c, c->d.bgx, bx)) || (rc = upload(c, c->d.bgy, by)) ||
       (rc = upload(c, c->d.eb0, e0)) || (rc = upload(c, c->d.eb1, e1)) ||
-      (rc = upload_form(c, c->d.bgR, bg, 2, true)))
+      (rc = upload_form(c, c->d.bgR, bg, 1, false)))
     return rc;
   return 0;
 }
@@ -1145,8 +1181,9 @@ void launch_gate(gks2l_ctx *c, const Par &p, cudaStream_t st) {
 template <typename R>
 void launch_recon(gks2l_ctx *c, const Par &p) {
   const Dev &d = c->d;
-  if (p.pos_floor > 0) k_recon<R, true><<<blocks(d.nt, TW), dim3(TW, 6), recon_smem<R>(), c->stream>>>(d, p);
-  else k_recon<R><<<blocks(d.nt, TW), dim3(TW, 6), recon_smem<R>(), c->stream>>>(d, p);
+  const dim3 block(TW, 6 / ReconCfg<R>::VP);
+  if (p.pos_floor > 0) k_recon<R, true><<<blocks(d.nt, TW), block, recon_smem<R>(), c->stream>>>(d, p);
+  else k_recon<R><<<blocks(d.nt, TW), block, recon_smem<R>(), c->stream>>>(d, p);
 }
 
 // launch shapes the autotuner chooses from: 0: 64 threads, 1: 128 threads,
@@ -1410,12 +1447,14 @@ int gks2l_bind(gks2l_ctx *c, void *d_workspace, size_t bytes, void *stream) {
   const Prep &P = c->prep;
   const int nt = P.nt;
   std::vector<double> fsl(3 * (size_t)nt), en(2 * (size_t)P.ne), ihs(nt), epsA(nt);
+  std::vector<int> txf(c->cs / TW, 0);
   for (int j = 0; j < nt; j++) {
     for (int f = 0; f < 3; f++) {
       int ce = P.cedge[f * nt + j];
       int e = ce >= 0 ? ce : ~ce;
       fsl[f * nt + j] = (ce >= 0 ? 1.0 : -1.0) * P.elen[e] / P.area[j];
     }
+    for (int r = 0; r < kSlots; r++) txf[j / TW] |= P.st_xf[(size_t)r * nt + j] != 0;
     ihs[j] = 1.0 / P.hs[j];
     epsA[j] = c->par.weno_eps * P.area[j];
   }
@@ -1426,7 +1465,7 @@ int gks2l_bind(gks2l_ctx *c, void *d_workspace, size_t bytes, void *stream) {
   if ((rc = upload(c, c->d.inst, P.inst)) || (rc = upload(c, c->d.area, P.area)) ||
       (rc = upload(c, c->d.hs, P.hs)) || (rc = upload(c, c->d.dX, P.dX)) ||
       (rc = upload_rows<int>(c, c->d.st_cell, P.st_cell, kSlots)) ||
-      (rc = upload_rows<int8_t>(c, c->d.st_xf, P.st_xf, kSlots)) ||
+      (rc = upload_rows<int8_t>(c, c->d.st_xf, P.st_xf, kSlots)) || (rc = upload(c, c->d.tile_xf, txf)) ||
       (rc = upload_rows<int>(c, c->d.cedge, P.cedge, 3)) || (rc = upload_rows<double>(c, c->d.fsl, fsl, 3)) ||
       (rc = upload_form(c, c->d.fslR, fsl, 3, true)) ||
       (rc = upload(c, c->d.inst_first, P.inst_first)) || (rc = upload(c, c->d.eL, P.eL)) ||

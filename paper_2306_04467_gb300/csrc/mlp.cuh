@@ -34,33 +34,35 @@ struct alignas(16) MlpDev {
 // mean and the h-scaled gradient, divided by the norm of all twelve
 // (regularised by the WENO epsilon, so smooth data give small features).
 template <typename R>
-__host__ __device__ inline void gate_features(const Dev &d, int j, const int *st, const int8_t *sx, int S, int I,
-                                              float out[24]) {
-  int nb[3], xf[3];
+__host__ __device__ inline void gate_features(const Dev &d, int j, float out[24]) {
+  // the levels' pair (h2, eta1) of the cell and its face neighbours: one load
+  // for a cell's two averages and one for their gradients
+  R q[4][2], g[4][4];
+  load_n<R, 2>(dq_at<R>(d, 0, j), q[0]);
+  load_g<R>(d, 0, j, g[0]);
+  int xf[3];
   for (int f = 0; f < 3; f++) {
-    nb[f] = st[f * S + I];
-    xf[f] = sx[f * S + I];
+    const int nb = d.st_cell[(size_t)f * d.cs + j];
+    xf[f] = d.st_xf[(size_t)f * d.cs + j];
+    load_n<R, 2>(dq_at<R>(d, 0, nb), q[1 + f]);
+    load_g<R>(d, 0, nb, g[1 + f]);
   }
+  for (int f = 0; f < 3; f++) image_g<R>(d, 0, xf[f], g[1 + f]);
   const R hs = ((const R *)d.hsR)[j];
   const R eps = ((const R *)d.epsA)[j];
+  R ref[2];
+  load_n<R, 2>((const R *)d.refR + 2 * d.inst[j], ref);
   for (int h = 0; h < 2; h++) {
-    const int v = h == 0 ? 3 : 0;
-    R q[4], g[4][2];
-    q[0] = ((const R *)d.dq)[v * d.cs + j];
-    img_dg<R>(d, v, j, 0, g[0]);
-    for (int f = 0; f < 3; f++) {
-      q[1 + f] = img_dq<R>(d, v, nb[f], xf[f]);
-      img_dg<R>(d, v, nb[f], xf[f], g[1 + f]);
-    }
-    R mean = (q[0] + q[1] + q[2] + q[3]) * (R)0.25;
+    const int c = 1 - h;
+    R mean = (q[0][c] + q[1][c] + q[2][c] + q[3][c]) * (R)0.25;
     R raw[12], ss = 0;
     for (int m = 0; m < 4; m++) {
-      raw[3 * m] = q[m] - mean;
-      raw[3 * m + 1] = hs * g[m][0];
-      raw[3 * m + 2] = hs * g[m][1];
+      raw[3 * m] = q[m][c] - mean;
+      raw[3 * m + 1] = hs * g[m][2 * c];
+      raw[3 * m + 2] = hs * g[m][2 * c + 1];
     }
     for (int k = 0; k < 12; k++) ss += raw[k] * raw[k];
-    R Q0 = q[0] + ((const R *)d.refR)[2 * d.inst[j] + (v == 3 ? 1 : 0)];
+    R Q0 = q[0][c] + ref[c];
     ss += eps * (1 + Q0 * Q0);
     R is = (R)1 / r_sqrt<R>(ss);
     for (int k = 0; k < 12; k++) out[12 * h + k] = (float)(raw[k] * is);

@@ -46,7 +46,12 @@ constexpr int NCOEF = 10;    // per variable: c0 (value offset) + 9 Taylor coeff
 // coefficients, the cell-average deviation, then a constant: 1/h_s in slot 0,
 // the bottom slope in slots 1-2 (lower layer; zero in the upper). An edge
 // point reads its layer's record and slot 0 (the level) of the other layer's.
-// 16-byte aligned, read with vector loads.
+// In memory the records of a tile of 32 cells are one block, vector by vector:
+// [tile][layer][16-byte vector][cell in tile]. A warp of the edge kernels asks
+// for the same vector of a few neighbouring cells at a time, so it finds
+// several of them in a 128-byte line where a record of its own lies in two
+// lines for itself: k_iface<float> 145 -> 123 us, k_edge<float> 333 -> 300 us
+// (1.04 M triangles; the fused k_edgef, bound by issue, 287 -> 295 us).
 constexpr int NREC = 36;
 
 // Device view of the workspace. R-typed arrays are stored as void* and cast.
@@ -58,10 +63,11 @@ struct Dev {
   const double *area, *hs, *dX;
   const void *hsR, *ihsR;   // sqrt|Omega| and its inverse, type R
   const void *epsA;         // weno_eps * |Omega|, type R
-  const void *bgR;          // [2][cell] grad B, type R
+  const void *bgR;          // [cell][2] grad B, type R
   const double *bmean, *bgx, *bgy;
   const int *st_cell;
   const int8_t *st_xf;
+  const int *tile_xf;       // per tile of 32 cells: whether any of its stencils has an image transform
   const void *ops;          // per tile of 32 cells: the reconstruction's operator rows
   const void *plane;        // [(f*2+d)][cell] plane operator, type R
   const int *cedge;         // [f][cell]: edge id, or ~edge when the cell is the R side
@@ -69,11 +75,11 @@ struct Dev {
   const void *fslR;         // the same, type R (the other residuals)
   const int *inst_first;
   double *avg;              // state averages [v][cell] (FP64)
-  void *dq, *dg;            // deviation mirrors [6][cell], gradients [12][cell], type R
+  void *dq, *dg;            // deviation mirrors [pair][cell][2] and gradients [pair][cell][2][2], type R
   void *hrefc;              // R1 - B_j per cell, type R
   double *Wn, *Ln, *Ltn;    // stage snapshot (FP64; L and L_t rows of the layer depths only)
   void *incR;               // [4][cell] stage-1 part of the stage-2 momentum increment, type R
-  void *srec;               // side records [layer][cell][NREC], type R (lower layer first)
+  void *srec;               // side records [tile][layer][vector][32][16 bytes], type R (lower layer first)
   void *omg;                // omega_H / gamma_H of eta1 [0] and h2 [1], type R
   const void *mlp;          // gate network, packed image (MlpDev)
   unsigned *gate_mask;      // per tile of 32 cells: bit i = cell i takes the linear weights
@@ -195,6 +201,8 @@ __host__ __device__ __forceinline__ long long dbits(double x) {
   return b;
 #endif
 }
+// whether an instance is still advancing (its dt, zero once it has stopped), off the FP64 pipe
+__host__ __device__ __forceinline__ bool running(const Dev &d, int inst) { return dbits(d.dt[inst]) > 0; }
 __host__ __device__ __forceinline__ bool finite_bits(double x) { return ((dbits(x) >> 52) & 0x7ff) != 0x7ff; }
 
 template <typename R>
@@ -218,44 +226,95 @@ __host__ __device__ __forceinline__ void rot2(const double *M, R v[2]) {
 }
 
 // ------------------------------------------------------------------ cell data
-// Deviation of reconstructed variable v of cell c seen through transform xf.
-template <typename R>
-__host__ __device__ __forceinline__ R img_dq(const Dev &d, int v, int c, int xf) {
-  const int N = d.cs;
-  const R *dq = (const R *)d.dq;
-  if (v == 0 || v == 3 || xf == 0) return dq[v * N + c];
-  int b = v < 3 ? 1 : 4;
-  R m[2] = {dq[b * N + c], dq[(b + 1) * N + c]};
-  rot2<R>(d.xf + 4 * xf, m);
-  return m[v - b];
+// The mirrors hold the variables in pairs, the levels (h2, eta1) and the two
+// layers' discharges (x, y): a thread that works on a pair gathers a cell's
+// two deviations by one load and their gradients by another, and a mirrored
+// discharge or its gradient tensor is at hand whole.
+constexpr int NPAIR = 3;
+__host__ __device__ __forceinline__ int pair_of(int v) { return v == 0 || v == 3 ? 0 : (v < 3 ? 1 : 2); }
+__host__ __device__ __forceinline__ int comp_of(int v) { return v == 0 || v == 3 ? v / 3 : (v < 3 ? v - 1 : v - 4); }
+__host__ __device__ __forceinline__ int var_of(int pair, int comp) {
+  return pair == 0 ? 3 * comp : (pair == 1 ? 1 : 4) + comp;
 }
-// gradient of reconstructed variable v of cell c seen through transform xf
-// (for v = 3 the water level's: the stored grad h1 plus the cell's grad B)
+// n consecutive values (n * sizeof(R) a multiple of their 8- or 16-byte load)
+template <typename R, int n> __host__ __device__ __forceinline__ void load_n(const R *p, R *w) {
+  for (int i = 0; i < n; i++) w[i] = p[i];
+}
+template <typename R, int n> __host__ __device__ __forceinline__ void store_n(R *p, const R *w) {
+  for (int i = 0; i < n; i++) p[i] = w[i];
+}
+#ifdef __CUDACC__
+template <> __device__ __forceinline__ void load_n<float, 2>(const float *p, float *w) {
+  const float2 t = *reinterpret_cast<const float2 *>(p);
+  w[0] = t.x; w[1] = t.y;
+}
+template <> __device__ __forceinline__ void load_n<float, 4>(const float *p, float *w) {
+  const float4 t = *reinterpret_cast<const float4 *>(p);
+  w[0] = t.x; w[1] = t.y; w[2] = t.z; w[3] = t.w;
+}
+template <> __device__ __forceinline__ void load_n<double, 2>(const double *p, double *w) {
+  const double2 t = *reinterpret_cast<const double2 *>(p);
+  w[0] = t.x; w[1] = t.y;
+}
+template <> __device__ __forceinline__ void load_n<double, 4>(const double *p, double *w) {
+  load_n<double, 2>(p, w);
+  load_n<double, 2>(p + 2, w + 2);
+}
+template <> __device__ __forceinline__ void store_n<float, 2>(float *p, const float *w) {
+  *reinterpret_cast<float2 *>(p) = make_float2(w[0], w[1]);
+}
+template <> __device__ __forceinline__ void store_n<float, 4>(float *p, const float *w) {
+  *reinterpret_cast<float4 *>(p) = make_float4(w[0], w[1], w[2], w[3]);
+}
+template <> __device__ __forceinline__ void store_n<double, 2>(double *p, const double *w) {
+  *reinterpret_cast<double2 *>(p) = make_double2(w[0], w[1]);
+}
+template <> __device__ __forceinline__ void store_n<double, 4>(double *p, const double *w) {
+  store_n<double, 2>(p, w);
+  store_n<double, 2>(p + 2, w + 2);
+}
+#endif
+template <typename R> __host__ __device__ __forceinline__ R *dq_at(const Dev &d, int pair, int c) {
+  return (R *)d.dq + ((size_t)pair * d.cs + c) * 2;
+}
+template <typename R> __host__ __device__ __forceinline__ R *dg_at(const Dev &d, int pair, int c) {
+  return (R *)d.dg + ((size_t)pair * d.cs + c) * 4;
+}
+
+// A pair's deviations (q) and gradients (g: of the first, then the second, the
+// level eta1's as stored plus the cell's grad B) seen through transform xf.
 template <typename R>
-__host__ __device__ __forceinline__ void img_dg(const Dev &d, int v, int c, int xf, R g[2]) {
-  const int N = d.cs;
-  const R *G = (const R *)d.dg;
-  if (v == 0 || v == 3 || xf == 0) {
-    g[0] = G[(2 * v) * N + c];
-    g[1] = G[(2 * v + 1) * N + c];
-    if (v == 3) {
-      g[0] += ((const R *)d.bgR)[c];
-      g[1] += ((const R *)d.bgR)[N + c];
-    }
-    if (xf != 0) rot2<R>(d.xf + 4 * xf, g);
+__host__ __device__ __forceinline__ void image_q(const Dev &d, int pair, int xf, R q[2]) {
+  if (pair != 0 && xf != 0) rot2<R>(d.xf + 4 * xf, q);
+}
+template <typename R>
+__host__ __device__ __forceinline__ void load_g(const Dev &d, int pair, int c, R g[4]) {
+  load_n<R, 4>(dg_at<R>(d, pair, c), g);
+  if (pair == 0) {
+    R b[2];
+    load_n<R, 2>((const R *)d.bgR + 2 * (size_t)c, b);
+    g[2] += b[0];
+    g[3] += b[1];
+  }
+}
+template <typename R>
+__host__ __device__ __forceinline__ void image_g(const Dev &d, int pair, int xf, R g[4]) {
+  if (xf == 0) return;
+  const double *M = d.xf + 4 * xf;
+  if (pair == 0) {
+    rot2<R>(M, g);
+    rot2<R>(M, g + 2);
     return;
   }
-  const double *M = d.xf + 4 * xf;
-  // discharge gradient tensor T_ik = d m_i / d x_k -> M T M^T, row v - b
-  int b = v < 3 ? 1 : 4;
-  int row = v - b;
-  R T[2][2] = {{G[(2 * b) * N + c], G[(2 * b + 1) * N + c]}, {G[(2 * b + 2) * N + c], G[(2 * b + 3) * N + c]}};
-  for (int k = 0; k < 2; k++) {
-    R s = 0;
-    for (int a = 0; a < 2; a++)
-      for (int b2 = 0; b2 < 2; b2++) s += (R)M[2 * row + a] * T[a][b2] * (R)M[2 * k + b2];
-    g[k] = s;
-  }
+  // discharge gradient tensor T_ik = d m_i / d x_k -> M T M^T
+  const R T[2][2] = {{g[0], g[1]}, {g[2], g[3]}};
+  for (int row = 0; row < 2; row++)
+    for (int k = 0; k < 2; k++) {
+      R s = 0;
+      for (int a = 0; a < 2; a++)
+        for (int b2 = 0; b2 < 2; b2++) s += (R)M[2 * row + a] * T[a][b2] * (R)M[2 * k + b2];
+      g[2 * row + k] = s;
+    }
 }
 
 // --------------------------------------------------- compact reconstruction
@@ -263,47 +322,114 @@ __host__ __device__ __forceinline__ void img_dg(const Dev &d, int v, int c, int 
 // (a tile staged in shared memory: stride = tile width, idx = cell in the tile).
 template <typename R> struct CellOps {
   const R *lsq, *p1, *bq, *mm;
-  const int *st;
-  const int8_t *sx;
   int stride, idx;
 };
 
-// One cell and one variable: P3 least squares (Eq. Recons-system), three P1
-// candidates on {cell, face neighbour}, smoothness indicators and WENO-Z
-// weights, combined polynomial written as deviations in the Taylor basis.
-// Three steps: gather the right-hand side, solve the P3 fit, then combine
-// (where the troubled-cell gate can choose the linear weights).
+// One cell and VP variables, a pair (VP = 2) or one of it (VP = 1, comp): P3
+// least squares (Eq. Recons-system), three P1 candidates on {cell, face
+// neighbour}, smoothness indicators and WENO-Z weights, combined polynomial
+// written as deviations in the Taylor basis. Three steps: gather the
+// right-hand side, solve the P3 fit, then combine (where the troubled-cell
+// gate can choose the linear weights).
 
 // right-hand side: stencil average differences, then h-scaled gradients of
-// the cell and its three face neighbours
+// the cell and its three face neighbours. st: the stencil's cells (-1: none);
+// xfs: whether any stencil of the tile is seen through a transform
 template <typename R>
-__host__ __device__ inline void recon_gather(const Dev &d, const CellOps<R> &o, int j, int v, R rhs[NCOL]) {
-  const int N = d.cs, S = o.stride, I = o.idx;
-  const R q0 = ((const R *)d.dq)[v * N + j];
+__host__ __device__ __forceinline__ void gather_one(const Dev &d, int j, int pair, int comp, const int st[NSLOT],
+                                                    bool xfs, R rhs[NCOL], R &q0) {
+  q0 = dq_at<R>(d, pair, j)[comp];
   const R hs = ((const R *)d.hsR)[j];
+#pragma unroll
   for (int s = 0; s < NSLOT; s++) {
-    int c = o.st[s * S + I];
-    rhs[s] = c >= 0 ? img_dq<R>(d, v, c, o.sx[s * S + I]) - q0 : (R)0;
+    const int c = st[s] >= 0 ? st[s] : j;
+    R t = dq_at<R>(d, pair, c)[comp];
+    const int xf = xfs && pair != 0 ? d.st_xf[(size_t)s * d.cs + j] : 0;
+    if (xf != 0) {
+      R m[2];
+      load_n<R, 2>(dq_at<R>(d, pair, c), m);
+      image_q<R>(d, pair, xf, m);
+      t = comp == 0 ? m[0] : m[1];
+    }
+    rhs[s] = st[s] >= 0 ? t - q0 : (R)0;
   }
-  R g[2];
-  img_dg<R>(d, v, j, 0, g);
-  rhs[9] = hs * g[0];
-  rhs[10] = hs * g[1];
-  for (int f = 0; f < 3; f++) {
-    img_dg<R>(d, v, o.st[f * S + I], o.sx[f * S + I], g);
-    rhs[11 + 2 * f] = hs * g[0];
-    rhs[12 + 2 * f] = hs * g[1];
+#pragma unroll
+  for (int m = 0; m < 4; m++) {
+    const int c = m == 0 ? j : st[m - 1];
+    R g[2];
+    load_n<R, 2>(dg_at<R>(d, pair, c) + 2 * comp, g);
+    if (pair == 0 && comp == 1) {
+      R b[2];
+      load_n<R, 2>((const R *)d.bgR + 2 * (size_t)c, b);
+      g[0] += b[0];
+      g[1] += b[1];
+    }
+    const int xf = xfs && m > 0 ? d.st_xf[(size_t)(m - 1) * d.cs + j] : 0;
+    if (xf != 0) {
+      if (pair == 0) {
+        rot2<R>(d.xf + 4 * xf, g);
+      } else {
+        R T[4];
+        load_n<R, 4>(dg_at<R>(d, pair, c), T);
+        image_g<R>(d, pair, xf, T);
+        g[0] = comp == 0 ? T[0] : T[2];
+        g[1] = comp == 0 ? T[1] : T[3];
+      }
+    }
+    rhs[9 + 2 * m] = hs * g[0];
+    rhs[10 + 2 * m] = hs * g[1];
+  }
+}
+template <typename R, int VP>
+__host__ __device__ __forceinline__ void recon_gather(const Dev &d, int j, int pair, int comp, const int st[NSLOT],
+                                                      bool xfs, R rhs[VP][NCOL], R q0[VP]) {
+  if (VP == 1) {
+    gather_one<R>(d, j, pair, comp, st, xfs, rhs[0], q0[0]);
+    return;
+  }
+  R q[2], t[NSLOT][2], g[4][4];
+  load_n<R, 2>(dq_at<R>(d, pair, j), q);
+#pragma unroll
+  for (int s = 0; s < NSLOT; s++) load_n<R, 2>(dq_at<R>(d, pair, st[s] >= 0 ? st[s] : j), t[s]);
+  load_g<R>(d, pair, j, g[0]);
+#pragma unroll
+  for (int f = 0; f < 3; f++) load_g<R>(d, pair, st[f], g[1 + f]);
+  const R hs = ((const R *)d.hsR)[j];
+  if (xfs) {
+#pragma unroll
+    for (int s = 0; s < NSLOT; s++) {
+      const int xf = d.st_xf[(size_t)s * d.cs + j];
+      image_q<R>(d, pair, xf, t[s]);
+      if (s < 3) image_g<R>(d, pair, xf, g[1 + s]);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < VP; i++) {
+    q0[i] = q[i];
+#pragma unroll
+    for (int s = 0; s < NSLOT; s++) rhs[i][s] = st[s] >= 0 ? t[s][i] - q0[i] : (R)0;
+#pragma unroll
+    for (int m = 0; m < 4; m++) {
+      rhs[i][9 + 2 * m] = hs * g[m][2 * i];
+      rhs[i][10 + 2 * m] = hs * g[m][2 * i + 1];
+    }
   }
 }
 
-// P3 least-squares coefficients a = M rhs
-template <typename R>
-__host__ __device__ inline void recon_p3(const CellOps<R> &o, const R rhs[NCOL], R a[9]) {
+// P3 least-squares coefficients a = M rhs; each operator entry is read once
+// for the thread's variables
+template <typename R, int VP>
+__host__ __device__ __forceinline__ void recon_p3(const CellOps<R> &o, const R rhs[VP][NCOL], R a[VP][9]) {
   const int S = o.stride, I = o.idx;
+#pragma unroll
   for (int r = 0; r < 9; r++) {
-    R s = 0;
-    for (int c = 0; c < NCOL; c++) s += o.lsq[(r * NCOL + c) * S + I] * rhs[c];
-    a[r] = s;
+    R s[VP] = {};
+#pragma unroll
+    for (int c = 0; c < NCOL; c++) {
+      const R m = o.lsq[(r * NCOL + c) * S + I];
+      for (int i = 0; i < VP; i++) s[i] += m * rhs[i][c];
+    }
+    for (int i = 0; i < VP; i++) a[i][r] = s[i];
   }
 }
 
@@ -324,107 +450,141 @@ __host__ __device__ __forceinline__ void ratios2(R t, R a, R b, R r[2]) {
   }
 }
 
-// The result goes to the cell's side records: straight to global memory, or,
-// with `stage` set, to a block's staging tile [layer][cell in tile][NREC]
-// (o.stride cells per layer) that the block then writes out with 16-byte
-// stores.
-template <typename R>
-__host__ __device__ inline void recon_finish(const Dev &d, const Par &p, const CellOps<R> &o, int j, int v,
-                                             const R rhs[NCOL], const R a[9], bool linear, R *stage = nullptr) {
+// The variables' slots of the side records (12 values each, see NREC).
+template <typename R, int VP>
+__host__ __device__ __forceinline__ void recon_finish(const Dev &d, const Par &p, const CellOps<R> &o, int j, int pair,
+                                                      int comp, const R rhs[VP][NCOL], const R a[VP][9],
+                                                      const R q0[VP], bool linear, R rec[VP][12]) {
   const int N = d.cs, S = o.stride, I = o.idx;
-  const R q0 = ((const R *)d.dq)[v * N + j];
   const R gh = pv<R>(p.gam_hi, p.gam_hif), gl = ((R)1 - gh) * (R)(1.0 / 3.0);
-  R fac = 1, wf[3] = {gl, gl, gl}, b[3][2] = {{0, 0}, {0, 0}, {0, 0}};
-  if (!linear) {
-    R beta[4];
+  R fac[VP], wf[VP][3], b[VP][3][2];
+  for (int i = 0; i < VP; i++) {
+    fac[i] = 1;
     for (int f = 0; f < 3; f++) {
-      R r5[5] = {rhs[f], rhs[9], rhs[10], rhs[11 + 2 * f], rhs[12 + 2 * f]};
+      wf[i][f] = gl;
+      b[i][f][0] = b[i][f][1] = 0;
+    }
+  }
+  if (!linear) {
+    R beta[VP][4], bh[VP] = {};
+#pragma unroll
+    for (int f = 0; f < 3; f++) {
+#pragma unroll
       for (int k = 0; k < 2; k++) {
-        R s = 0;
-        for (int c = 0; c < 5; c++) s += o.p1[((f * 2 + k) * 5 + c) * S + I] * r5[c];
-        b[f][k] = s;
+        R s[VP] = {};
+#pragma unroll
+        for (int c = 0; c < 5; c++) {
+          const R m = o.p1[((f * 2 + k) * 5 + c) * S + I];
+          const int col = c == 0 ? f : (c < 3 ? 8 + c : 8 + 2 * f + c);
+          for (int i = 0; i < VP; i++) s[i] += m * rhs[i][col];
+        }
+        for (int i = 0; i < VP; i++) b[i][f][k] = s[i];
       }
-      beta[1 + f] = b[f][0] * b[f][0] + b[f][1] * b[f][1];
+      for (int i = 0; i < VP; i++) beta[i][1 + f] = b[i][f][0] * b[i][f][0] + b[i][f][1] * b[i][f][1];
     }
-    R bh = 0;
     int idx = 0;
+#pragma unroll
     for (int k = 0; k < 9; k++) {
-      if (sizeof(R) == 8) {
-        // a_k times the row's sum: 54 operations in place of 90 (with the
-        // weights' shared reciprocals k_recon<double> goes from 404 to 344 FP64
-        // operations per cell and variable, 2224 -> 1897 us at 501 k triangles)
-        R row = 0;
-        for (int l = k; l < 9; l++) row += o.bq[(idx++) * S + I] * a[l];
-        bh += a[k] * row;
-      } else {
-        for (int l = k; l < 9; l++) bh += o.bq[(idx++) * S + I] * a[k] * a[l];
-      }
-    }
-    beta[0] = bh;
-    R tz = (r_abs<R>(bh - beta[1]) + r_abs<R>(bh - beta[2]) + r_abs<R>(bh - beta[3])) * (R)(1.0 / 3.0);
-    // the variable's value (reference + deviation) scales the regulariser
-    R Q0 = q0;
-    const R *refR = (const R *)d.refR;
-    if (v == 0) Q0 += refR[2 * d.inst[j]];
-    if (v == 3) Q0 += refR[2 * d.inst[j] + 1];
-    R eps = ((const R *)d.epsA)[j] * (1 + Q0 * Q0);
-    const R gam[4] = {gh, gl, gl, gl};
-    if (sizeof(R) == 8) {
-      R u[4], ws = 0;
-      for (int k = 0; k < 4; k += 2) {
-        R r[2];
-        ratios2<R>(tz, beta[k] + eps, beta[k + 1] + eps, r);
-        for (int i = 0; i < 2; i++) {
-          u[k + i] = 1 + r[i] * r[i];
-          ws += gam[k + i] * u[k + i];
+      R row[VP] = {};
+#pragma unroll
+      for (int l = k; l < 9; l++) {
+        const R m = o.bq[(idx++) * S + I];
+        for (int i = 0; i < VP; i++) {
+          // double form: a_k times the row's sum, 54 operations in place of 90
+          // (with the weights' shared reciprocals k_recon<double> goes from
+          // 404 to 344 FP64 operations per cell and variable, 2224 -> 1897 us
+          // at 501 k triangles)
+          if (sizeof(R) == 8) row[i] += m * a[i][l];
+          else bh[i] += m * a[i][k] * a[i][l];
         }
       }
-      const R iw = 1 / ws;
-      fac = u[0] * iw;
-      for (int f = 0; f < 3; f++) wf[f] = u[1 + f] * (gl * iw);
-    } else {
-      R w[4], ws = 0;
-      for (int k = 0; k < 4; k++) {
-        R r = tz / (beta[k] + eps);
-        w[k] = gam[k] * (1 + r * r);
-        ws += w[k];
-      }
-      R iw = 1 / ws;
-      fac = w[0] * iw / gh;
-      for (int f = 0; f < 3; f++) wf[f] = w[1 + f] * iw;
+      if (sizeof(R) == 8)
+        for (int i = 0; i < VP; i++) bh[i] += a[i][k] * row[i];
     }
-    if (p.harvest) {
-      R dv = r_abs<R>(fac - 1);
-      for (int f = 0; f < 3; f++) {
-        R df = r_abs<R>(wf[f] / gl - 1);
-        dv = df > dv ? df : dv;
+    const R gam[4] = {gh, gl, gl, gl};
+    const R epsA = ((const R *)d.epsA)[j];
+    const int in = d.inst[j];
+#pragma unroll
+    for (int i = 0; i < VP; i++) {
+      const int c = VP == 2 ? i : comp;
+      beta[i][0] = bh[i];
+      R tz = (r_abs<R>(bh[i] - beta[i][1]) + r_abs<R>(bh[i] - beta[i][2]) + r_abs<R>(bh[i] - beta[i][3])) *
+             (R)(1.0 / 3.0);
+      // the variable's value (reference + deviation) scales the regulariser
+      R Q0 = q0[i];
+      if (pair == 0) Q0 += ((const R *)d.refR)[2 * in + c];
+      R eps = epsA * (1 + Q0 * Q0);
+      if (sizeof(R) == 8) {
+        R u[4], ws = 0;
+        for (int k = 0; k < 4; k += 2) {
+          R r[2];
+          ratios2<R>(tz, beta[i][k] + eps, beta[i][k + 1] + eps, r);
+          for (int m = 0; m < 2; m++) {
+            u[k + m] = 1 + r[m] * r[m];
+            ws += gam[k + m] * u[k + m];
+          }
+        }
+        const R iw = 1 / ws;
+        fac[i] = u[0] * iw;
+        for (int f = 0; f < 3; f++) wf[i][f] = u[1 + f] * (gl * iw);
+      } else {
+        R w[4], ws = 0;
+        for (int k = 0; k < 4; k++) {
+          R r = tz / (beta[i][k] + eps);
+          w[k] = gam[k] * (1 + r * r);
+          ws += w[k];
+        }
+        R iw = 1 / ws;
+        fac[i] = w[0] * iw / gh;
+        for (int f = 0; f < 3; f++) wf[i][f] = w[1 + f] * iw;
       }
-      d.wdev[v * N + j] = (float)dv;
+      if (p.harvest) {
+        R dv = r_abs<R>(fac[i] - 1);
+        for (int f = 0; f < 3; f++) {
+          R df = r_abs<R>(wf[i][f] / gl - 1);
+          dv = df > dv ? df : dv;
+        }
+        d.wdev[(size_t)var_of(pair, c) * N + j] = (float)dv;
+      }
     }
   } else if (p.harvest) {
-    d.wdev[v * N + j] = 0.f;
+    for (int i = 0; i < VP; i++) d.wdev[(size_t)var_of(pair, VP == 2 ? i : comp) * N + j] = 0.f;
   }
   // R = (w_H / g_H)(P3 - sum g_m P1_m) + sum w_m P1_m
-  R r[10];
-  for (int k = 1; k < 10; k++) r[k] = fac * a[k - 1];
-  for (int f = 0; f < 3; f++) {
-    R cf = wf[f] - fac * gl;
-    r[1] += cf * b[f][0];
-    r[2] += cf * b[f][1];
+#pragma unroll
+  for (int i = 0; i < VP; i++) {
+    R *r = rec[i];
+    for (int k = 1; k < 10; k++) r[k] = fac[i] * a[i][k - 1];
+    for (int f = 0; f < 3; f++) {
+      R cf = wf[i][f] - fac[i] * gl;
+      r[1] += cf * b[i][f][0];
+      r[2] += cf * b[i][f][1];
+    }
+    r[0] = 0;
+    r[10] = q0[i];
+    // omega_H / gamma_H of eta1, then of h2
+    if (pair == 0) ((R *)d.omg)[(size_t)((VP == 2 ? i : comp) == 1 ? 0 : N) + j] = fac[i];
   }
-  R c0 = 0;
-  for (int k = 3; k < 10; k++) c0 -= r[k] * o.mm[(k - 3) * S + I];
-  r[0] = c0;
-  // the layer's side record (vars 3,4,5 -> lower, 0,1,2 -> upper), and the
-  // other layer's record for the level variables 0 and 3
-  R *rec = stage ? stage : (R *)d.srec;
-  const size_t ncell = stage ? (size_t)S : (size_t)N, cell = stage ? (size_t)I : (size_t)j;
-  const int rs = NREC;
-  R *p0 = rec + ((size_t)(v >= 3 ? 0 : 1) * ncell + cell) * rs + (v % 3) * 12;
-  for (int k = 0; k < 10; k++) p0[k] = r[k];
-  p0[10] = q0;
-  if (v == 3) ((R *)d.omg)[j] = fac;
-  if (v == 0) ((R *)d.omg)[N + j] = fac;
+#pragma unroll
+  for (int k = 3; k < 10; k++) {
+    const R m = o.mm[(k - 3) * S + I];
+    for (int i = 0; i < VP; i++) rec[i][0] -= rec[i][k] * m;
+  }
+  // the slots' constants: 1/h_s with the level, the bottom slope with the
+  // lower layer's discharges
+  if (pair == 0) {
+    const R ih = ((const R *)d.ihsR)[j];
+    for (int i = 0; i < VP; i++) rec[i][11] = ih;
+  } else {
+    R g[2] = {0, 0};
+    if (pair == 2) load_n<R, 2>((const R *)d.bgR + 2 * (size_t)j, g);
+    for (int i = 0; i < VP; i++) rec[i][11] = (VP == 2 ? i : comp) == 0 ? g[0] : g[1];
+  }
+}
+// layer (0 lower) and slot of a variable's part of the side records
+__host__ __device__ __forceinline__ int slot_of(int pair, int comp, int &layer) {
+  layer = pair == 0 ? 1 - comp : (pair == 2 ? 0 : 1);
+  return pair == 0 ? 0 : 1 + comp;
 }
 
 // ------------------------------------------------- evaluation at an edge point
@@ -442,44 +602,22 @@ template <typename R> struct SideVals {
 
 // cell c's reconstruction at scaled point (x, y), seen through transform xf;
 // href is the depth of the reference level at the point
-// n consecutive values of a side record (n a multiple of 4)
-template <typename R, int n> __host__ __device__ __forceinline__ void load_rec(const R *p, R *w) {
-  for (int k = 0; k < n; k++) w[k] = p[k];
-}
-#ifdef __CUDACC__
-template <> __device__ __forceinline__ void load_rec<float, NREC>(const float *p, float *w) {
-  const float4 *q = reinterpret_cast<const float4 *>(p);
+// the first n values (a multiple of 12) of cell c's side record of layer ell
+constexpr int RTILE = 32;    // cells per tile of the side records
+template <typename R, int n>
+__host__ __device__ __forceinline__ void load_rec(const Dev &d, int ell, int c, R *w) {
+  constexpr int V = 16 / sizeof(R);   // values per vector
+  const R *p = (const R *)d.srec + ((size_t)((unsigned)c / RTILE) * 2 + ell) * (NREC * RTILE) + ((unsigned)c % RTILE) * V;
 #pragma unroll
-  for (int k = 0; k < NREC / 4; k++) {
-    float4 t = q[k];
-    w[4 * k] = t.x; w[4 * k + 1] = t.y; w[4 * k + 2] = t.z; w[4 * k + 3] = t.w;
-  }
-}
-template <> __device__ __forceinline__ void load_rec<float, 12>(const float *p, float *w) {
-  const float4 *q = reinterpret_cast<const float4 *>(p);
-#pragma unroll
-  for (int k = 0; k < 3; k++) {
-    float4 t = q[k];
-    w[4 * k] = t.x; w[4 * k + 1] = t.y; w[4 * k + 2] = t.z; w[4 * k + 3] = t.w;
-  }
-}
-template <> __device__ __forceinline__ void load_rec<double, NREC>(const double *p, double *w) {
-  const double2 *q = reinterpret_cast<const double2 *>(p);
-#pragma unroll
-  for (int k = 0; k < NREC / 2; k++) {
-    double2 t = q[k];
-    w[2 * k] = t.x; w[2 * k + 1] = t.y;
-  }
-}
-template <> __device__ __forceinline__ void load_rec<double, 12>(const double *p, double *w) {
-  const double2 *q = reinterpret_cast<const double2 *>(p);
-#pragma unroll
-  for (int k = 0; k < 6; k++) {
-    double2 t = q[k];
-    w[2 * k] = t.x; w[2 * k + 1] = t.y;
-  }
-}
+  for (int k = 0; k < n / V; k++) {
+#ifdef __CUDA_ARCH__
+    const uint4 t = *reinterpret_cast<const uint4 *>(p + k * RTILE * V);
+    *reinterpret_cast<uint4 *>(w + k * V) = t;
+#else
+    for (int i = 0; i < V; i++) w[k * V + i] = p[k * RTILE * V + i];
 #endif
+  }
+}
 
 // Operations rounded as written, whatever the compiler does with the code
 // around them: where two kernels must form the same value bit for bit.
@@ -544,9 +682,8 @@ __host__ __device__ __forceinline__ void rot2_rn(const double *M, R v[2]) {
 // that forms it as its own).
 template <typename R, bool OTHER = true>
 __host__ __device__ inline void side_vals(const Dev &d, int ell, int c, int xf, R x, R y, R href, SideVals<R> &s) {
-  const int N = d.cs;
   R w[NREC];
-  load_rec<R, NREC>((const R *)d.srec + ((size_t)ell * N + c) * NREC, w);
+  load_rec<R, NREC>(d, ell, c, w);
   R m[10], mx[10], my[10];
   monos<R>(x, y, m, mx, my);
   const R ih = w[11];
@@ -572,7 +709,7 @@ __host__ __device__ inline void side_vals(const Dev &d, int ell, int c, int xf, 
   s.goth[0] = s.goth[1] = 0;
   if (OTHER) {
     R wo[12];
-    load_rec<R, 12>((const R *)d.srec + ((size_t)(1 - ell) * N + c) * NREC, wo);
+    load_rec<R, 12>(d, 1 - ell, c, wo);
     level_grad<R>(wo, mx, my, ih, s.goth);
   }
   s.d = w[10] + dev[0];
@@ -860,18 +997,18 @@ __host__ __device__ __forceinline__ R blend_level(R dl, R hl, R mxl, R myl, R dr
 // points.
 template <typename R>
 __host__ __device__ inline R iface_unit(const Dev &d, int e, int ell) {
-  const int NE = d.ne, N = d.cs;
+  const int NE = d.ne;
   const R *xl = (const R *)d.exiL, *xr = (const R *)d.exiR, *en = (const R *)d.en;
   const int cL = d.eL[e], cR = d.eR[e], xf = d.exf[e];
   R vl[2][3], vr[2][3];
   {
     R w[NREC];
-    load_rec<R, NREC>((const R *)d.srec + ((size_t)ell * N + cL) * NREC, w);
+    load_rec<R, NREC>(d, ell, cL, w);
     for (int q = 0; q < 2; q++) rec_values<R>(w, xl[(2 * q) * NE + e], xl[(2 * q + 1) * NE + e], vl[q]);
   }
   {
     R w[NREC];
-    load_rec<R, NREC>((const R *)d.srec + ((size_t)ell * N + cR) * NREC, w);
+    load_rec<R, NREC>(d, ell, cR, w);
     for (int q = 0; q < 2; q++) rec_values<R>(w, xr[(2 * q) * NE + e], xr[(2 * q + 1) * NE + e], vr[q]);
   }
   const R n0 = en[e], n1 = en[NE + e];
@@ -994,7 +1131,10 @@ __host__ __device__ inline bool edge_unit(const Dev &d, const Par &p, int e, int
       R un[2], ut[2];
       for (int sd = 0; sd < 2; sd++) {
         const int c = sd == 0 ? cL : cR, x = sd == 0 ? 0 : xf;
-        const R mx = img_dq<R>(d, vm, c, x), my = img_dq<R>(d, vm + 1, c, x);
+        R m[2];
+        load_n<R, 2>(dq_at<R>(d, pair_of(vm), c), m);
+        image_q<R>(d, pair_of(vm), x, m);
+        const R mx = m[0], my = m[1];
         const R ih = (R)1 / hb[ell * N + c];
         un[sd] = (mx * n0 + my * n1) * ih;
         ut[sd] = (-mx * n1 + my * n0) * ih;
@@ -1104,8 +1244,9 @@ __host__ __device__ inline double update_unit(const Dev &d, const Par &p, int j,
     }
   }
   const R G = pv<R>(p.g, p.gf), chi = pv<R>(p.chi, p.chif);
-  const R gb[2] = {((const R *)d.bgR)[j], ((const R *)d.bgR)[N + j]};
-  const R *dq = (const R *)d.dq;
+  R gb[2], dq0[2];   // the levels' deviations (h2, eta1)
+  load_n<R, 2>((const R *)d.bgR + 2 * (size_t)j, gb);
+  load_n<R, 2>(dq_at<R>(d, 0, j), dq0);
   const R R2 = ((const R *)d.refR)[2 * in];
   const R hrc = ((const R *)d.hrefc)[j];          // R1 - B_j
   const R m1 = hrc + mO[0], m2 = R2 + mO[1];       // means of h1, h2 over the 6 Gauss points
@@ -1114,10 +1255,10 @@ __host__ __device__ inline double update_unit(const Dev &d, const Par &p, int j,
   for (int k = 0; k < 2; k++) {
     // upper layer: -G h2 grad(B + h1) with h1 = eta1 - B at the points; the
     // time derivative by the product rule with the interface solution's W_t (R4)
-    L[1 + k] = LF[1 + k] - G * (dq[j] - mO[1]) * gb[k] - G * m2 * GO[0][k];
+    L[1 + k] = LF[1 + k] - G * (dq0[0] - mO[1]) * gb[k] - G * m2 * GO[0][k];
     Lt[1 + k] = LFt[1 + k] - G * (LFh2 - mWt[0]) * gb[k] - G * mWt[0] * GO[0][k] - G * m2 * GGt[3][k];
     // lower layer: flux reference pressure + bottom source -> -G (eta1 - R1) grad B; interlayer -chi G h1 grad h2
-    L[4 + k] = LF[4 + k] - G * dq[3 * N + j] * gb[k] - chi * G * m1 * GO[1][k];
+    L[4 + k] = LF[4 + k] - G * dq0[1] * gb[k] - chi * G * m1 * GO[1][k];
     Lt[4 + k] = LFt[4 + k] - G * LFh1 * gb[k] - chi * G * (mWt[3] * GO[1][k] + m1 * GGt[0][k]);
   }
   // S2O4 (Eq. SWE-fully-discrete): stage 1 W* = W^n + dt/2 L^n + dt^2/8 L_t^n;
@@ -1157,16 +1298,21 @@ __host__ __device__ inline double update_unit(const Dev &d, const Par &p, int j,
     }
   }
   if (act) {
-    R *dqw = (R *)d.dq, *dgw = (R *)d.dg;
-    for (int v = 0; v < NV; v++) {
-      d.avg[v * N + j] = nw[v];
-      // the interface values of variable 3 are water levels: grad h1 = grad eta1 - grad B
-      dgw[(2 * v) * N + j] = v == 3 ? GGn[v][0] - gb[0] : GGn[v][0];
-      dgw[(2 * v + 1) * N + j] = v == 3 ? GGn[v][1] - gb[1] : GGn[v][1];
+    for (int v = 0; v < NV; v++) d.avg[v * N + j] = nw[v];
+    const R q[NPAIR][2] = {{(R)(nw[0] - d.ref[2 * in]), (R)((nw[3] + d.bmean[j]) - d.ref[2 * in + 1])},
+                           {(R)nw[1], (R)nw[2]},
+                           {(R)nw[4], (R)nw[5]}};
+    for (int i = 0; i < NPAIR; i++) {
+      const int v0 = var_of(i, 0), v1 = var_of(i, 1);
+      R g[4] = {GGn[v0][0], GGn[v0][1], GGn[v1][0], GGn[v1][1]};
+      if (i == 0) {
+        // the interface values of variable 3 are water levels: grad h1 = grad eta1 - grad B
+        g[2] -= gb[0];
+        g[3] -= gb[1];
+      }
+      store_n<R, 2>(dq_at<R>(d, i, j), q[i]);
+      store_n<R, 4>(dg_at<R>(d, i, j), g);
     }
-    dqw[j] = (R)(nw[0] - d.ref[2 * in]);
-    dqw[3 * N + j] = (R)((nw[3] + d.bmean[j]) - d.ref[2 * in + 1]);
-    for (int i = 0; i < 4; i++) dqw[mom[i] * N + j] = (R)nw[mom[i]];
   }
   // health flags by integer tests on the bits (off the FP64 pipe)
   int fl = 0;
