@@ -200,7 +200,8 @@ __global__ void __launch_bounds__(TW * 6 / ReconCfg<R>::VP, ReconCfg<R>::BLOCKS)
   // the stencil's values and the cell's activity (a chain of two loads)
   // arrive beside the copies
   const int j = j0 + lane, jj = min(j, d.nt - 1);
-  const int pair = VP == 2 ? threadIdx.y : pair_of(threadIdx.y), comp = VP == 2 ? 0 : comp_of(threadIdx.y);
+  const int unit = blockIdx.y * blockDim.y + threadIdx.y;   // pair or variable
+  const int pair = VP == 2 ? unit : pair_of(unit), comp = VP == 2 ? 0 : comp_of(unit);
   const bool active = j < d.nt && (p.all_active || running(d, d.inst[jj]));
   R rhs[VP][NCOL], a[VP][9], q0[VP], rec[VP][12];
   auto gather = [&] {
@@ -233,7 +234,7 @@ __global__ void __launch_bounds__(TW * 6 / ReconCfg<R>::VP, ReconCfg<R>::BLOCKS)
   o.idx = lane;
   if (VP == 1) gather();
   const bool linear = ((lin_mask >> lane) & 1u) != 0;
-  if (gate_on && threadIdx.y == 0) {
+  if (gate_on && unit == 0) {
     const unsigned ns = __popc(__ballot_sync(FULL, active && linear)), nc = __popc(__ballot_sync(FULL, active));
     if (lane == 0) {
       atomicAdd(&d.gate_count[0], (unsigned long long)ns);
@@ -709,12 +710,12 @@ __global__ void __launch_bounds__(BS) k_edge(Dev d, Par p, int stage) { edge_bod
 // (the fused kernel's default shapes are held in FP32 to 768 resident threads
 // per SM, the 80 registers its body compiles to when left alone)
 template <typename R, int BS>
-__global__ void __launch_bounds__(BS, sizeof(R) == 4 ? 768 / BS : 1) k_edgef(Dev d, Par p, int stage) { edge_fused_body<R>(d, p, stage); }
+__global__ void __launch_bounds__(BS, sizeof(R) == 4 && BS > 32 ? 768 / BS : 1) k_edgef(Dev d, Par p, int stage) { edge_fused_body<R>(d, p, stage); }
 template <typename R, int BS>
 __global__ void __launch_bounds__(BS) k_update(Dev d, Par p, int stage) { update_body<R>(d, p, stage); }
 // the edge solution with the positivity option (one launch shape)
-template <typename R>
-__global__ void __launch_bounds__(128) k_edge_pos(Dev d, Par p, int stage) { edge_body<R, true>(d, p, stage); }
+template <typename R, int BS>
+__global__ void __launch_bounds__(BS) k_edge_pos(Dev d, Par p, int stage) { edge_body<R, true>(d, p, stage); }
 template <typename R>
 __global__ void __launch_bounds__(128, 8) k_iface_r64(Dev d) { iface_body<R>(d); }
 template <typename R>
@@ -1181,22 +1182,42 @@ void launch_gate(gks2l_ctx *c, const Par &p, cudaStream_t st) {
 template <typename R>
 void launch_recon(gks2l_ctx *c, const Par &p) {
   const Dev &d = c->d;
-  const dim3 block(TW, 6 / ReconCfg<R>::VP);
-  if (p.pos_floor > 0) k_recon<R, true><<<blocks(d.nt, TW), block, recon_smem<R>(), c->stream>>>(d, p);
-  else k_recon<R><<<blocks(d.nt, TW), block, recon_smem<R>(), c->stream>>>(d, p);
+  constexpr int UNITS = 6 / ReconCfg<R>::VP;
+  const unsigned tiles = blocks(d.nt, TW);
+  if (p.pos_floor > 0) {
+    k_recon<R, true><<<tiles, dim3(TW, UNITS), recon_smem<R>(), c->stream>>>(d, p);
+    return;
+  }
+  // a small mesh in FP64: a block per tile and variable, so that the tiles'
+  // warps share more SMs' FP64 pipes (each block fetches the tile's rows,
+  // from L2); from one tile per SM on all pipes have work anyway
+  const bool split = sizeof(R) == 8 && tiles < (unsigned)c->n_sm;
+  k_recon<R><<<dim3(tiles, split ? UNITS : 1), dim3(TW, split ? 1 : UNITS), recon_smem<R>(), c->stream>>>(d, p);
 }
 
 // launch shapes the autotuner chooses from: 0: 64 threads, 1: 128 threads,
 // 2: 256 threads (registers as the compiler likes), 3: 128 threads held to
-// 64 registers (eight blocks per SM), 4: 128 threads held to 128 registers
+// 64 registers (eight blocks per SM), 4: 128 threads held to 128 registers.
+// In shapes 0-2 a grid of the double form of fewer than kSpread 128-thread
+// blocks per SM takes blocks of one warp instead: the SMs' shares of the work,
+// bound by the FP64 pipe, then differ by one warp at most, not by four. With
+// the reconstruction's split, smooth flow on 512 triangles 87.5 -> 78.6 us a
+// stage, a queue of 5,000-triangle states 140 -> 130 us a stage; 65,522
+// triangles gain 0.3%, where the line is drawn. (In FP32 one-warp blocks are
+// slower: 122 -> 128 us for an exchange of 4,608 triangles.)
 constexpr int kShapes = 5;
+constexpr unsigned kSpread = 16;
+template <typename R> bool spread(const gks2l_ctx *c, size_t n) {
+  return sizeof(R) == 8 && blocks(n, 128) < kSpread * (unsigned)c->n_sm;
+}
 
 #define GKS2L_SHAPE_SWITCH(cfg, KERNEL, n, st, ...)                                          \
-  switch (cfg) {                                                                           \
+  switch (cfg < 3 && spread<R>(c, n) ? kShapes : cfg) {                                    \
     case 0: KERNEL<R, 64><<<blocks(n, 64), 64, 0, st>>>(__VA_ARGS__); break;                \
     case 2: KERNEL<R, 256><<<blocks(n, 256), 256, 0, st>>>(__VA_ARGS__); break;             \
     case 3: KERNEL##_r64<R><<<blocks(n, 128), 128, 0, st>>>(__VA_ARGS__); break;            \
     case 4: KERNEL##_r128<R><<<blocks(n, 128), 128, 0, st>>>(__VA_ARGS__); break;           \
+    case kShapes: KERNEL<R, 32><<<blocks(n, 32), 32, 0, st>>>(__VA_ARGS__); break;          \
     default: KERNEL<R, 128><<<blocks(n, 128), 128, 0, st>>>(__VA_ARGS__); break;            \
   }
 
@@ -1210,7 +1231,8 @@ template <typename R>
 void launch_edge(gks2l_ctx *c, const Par &p, int stage, cudaStream_t st) {
   const size_t n = 4 * (size_t)c->d.ne;
   if (p.pos_floor > 0) {
-    k_edge_pos<R><<<blocks(n, 128), 128, 0, st>>>(c->d, p, stage);
+    if (spread<R>(c, n)) k_edge_pos<R, 32><<<blocks(n, 32), 32, 0, st>>>(c->d, p, stage);
+    else k_edge_pos<R, 128><<<blocks(n, 128), 128, 0, st>>>(c->d, p, stage);
     return;
   }
   GKS2L_SHAPE_SWITCH(c->shape[1], k_edge, n, st, c->d, p, stage)
