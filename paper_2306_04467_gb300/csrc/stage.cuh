@@ -112,6 +112,7 @@ struct Dev {
   double *dt, *t;
   void *dtR;                // [2][inst] dt and 1/dt (0 for a stopped instance), type R
   unsigned long long *dtbits;
+  unsigned *ref_done;       // blocks of the reference-level reduction that have finished (wraps to 0)
   double *mass;             // [inst*2 + layer]
   int *status;
   unsigned long long *gate_count;
@@ -125,6 +126,7 @@ struct Par {
   int use_gate;                              // learned gate active
   float *logit_out;                          // gate logits per cell (device order), or null
   int all_active;                            // reconstruct every instance (harvesting)
+  int mask_now;                              // the gate writes the mask in use, not the next one
   int harvest;                               // record the weights' departure from linear
   int staging_polls;                         // > 0: operator staging polls at most this many - 1 times
   double pos_floor;                          // positivity option (not in the paper): 0 = off
