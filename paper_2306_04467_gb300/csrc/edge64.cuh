@@ -110,18 +110,19 @@ __host__ __device__ __forceinline__ double blend64(double dl, double ul, double 
 // iface_unit in the double form
 __host__ __device__ inline double iface_unit64(const Dev &d, int e, int ell) {
   using O = D64;
-  const int NE = d.ne;
-  const double *en = (const double *)d.en;
-  const double n0 = en[e], n1 = en[NE + e];
+  const EdgeIds g = edge_ids(d, e);
+  double x[2][4], n[2];
+  for (int q = 0; q < 2; q++) load_n<double, 4>((const double *)d.exi + ((size_t)q * d.ne + e) * 4, x[q]);
+  load_n<double, 2>((const double *)d.en + 2 * (size_t)e, n);
+  const double n0 = n[0], n1 = n[1];
   double lev[2][2], un[2][2];
   for (int sd = 0; sd < 2; sd++) {
-    const double *xs = sd == 0 ? (const double *)d.exiL : (const double *)d.exiR;
     double fr[4], w[NREC];
-    face_frame(d, n0, n1, sd == 0 ? 0 : d.exf[e], fr);
-    load_rec<double, NREC>(d, ell, sd == 0 ? d.eL[e] : d.eR[e], w);
+    face_frame(d, n0, n1, sd == 0 ? 0 : g.xf, fr);
+    load_rec<double, NREC>(d, ell, sd == 0 ? g.L : g.R, w);
     for (int q = 0; q < 2; q++) {
       double m[10];
-      monos64(xs[(2 * q) * NE + e], xs[(2 * q + 1) * NE + e], m);
+      monos64(x[q][2 * sd], x[q][2 * sd + 1], m);
       lev[sd][q] = poly_val64(w, m);
       const double r = r_rsqrt(O::add(ref_depth<double>(d, ell, e, q), lev[sd][q]));
       un[sd][q] = O::mul(O::fma(poly_val64(w + 12, m), fr[0], O::mul(poly_val64(w + 24, m), fr[1])), O::mul(r, r));
@@ -420,14 +421,16 @@ template <bool FUSED, bool PAIRED, bool POS>
 __host__ __device__ inline bool edge_unit64(const Dev &d, const Par &p, int e, int ell, int q, double out[12],
                                             double *blend, double *own) {
   using O = D64;
-  const int NE = d.ne;
-  const double *xl = (const double *)d.exiL, *xr = (const double *)d.exiR, *en = (const double *)d.en;
-  const int cL = d.eL[e], cR = d.eR[e], xf = d.exf[e], in = d.inst[cL];
+  const EdgeIds g = edge_ids(d, e);
+  const int cL = g.L, cR = g.R, xf = g.xf, in = g.inst;
+  double x[4], n[2];
+  load_n<double, 4>((const double *)d.exi + ((size_t)q * d.ne + e) * 4, x);
+  load_n<double, 2>((const double *)d.en + 2 * (size_t)e, n);
   // both stages fit the value and time derivative at their start from the
   // time integrals over dt and dt/2 (reading R20)
   const double dt = ((const double *)d.dtR)[in], idt = ((const double *)d.dtR)[d.ninst + in];
   const double href = ref_depth<double>(d, ell, e, q);
-  const double n0 = en[e], n1 = en[NE + e];
+  const double n0 = n[0], n1 = n[1];
   double fr[2][4], m[2][10];
   face_frame(d, n0, n1, 0, fr[0]);
   face_frame(d, n0, n1, xf, fr[1]);
@@ -437,14 +440,13 @@ __host__ __device__ inline bool edge_unit64(const Dev &d, const Par &p, int e, i
   constexpr bool SH = false;
 #endif
   if (!SH) {
-    monos64(xl[(2 * q) * NE + e], xl[(2 * q + 1) * NE + e], m[0]);
-    monos64(xr[(2 * q) * NE + e], xr[(2 * q + 1) * NE + e], m[1]);
+    monos64(x[0], x[1], m[0]);
+    monos64(x[2], x[3], m[1]);
   }
 #ifdef __CUDA_ARCH__
   if (SH) {
-    const double *xs = ell == 0 ? xl : xr;
     double mine[10];
-    monos64(xs[(2 * q) * NE + e], xs[(2 * q + 1) * NE + e], mine);
+    monos64(ell == 0 ? x[0] : x[2], ell == 0 ? x[1] : x[3], mine);
 #pragma unroll
     for (int k = 1; k < 10; k++) {
       const double theirs = __shfl_xor_sync(0xffffffffu, mine[k], 2);

@@ -140,13 +140,14 @@ template <typename R> constexpr unsigned recon_smem() { return TileLayout<R>::BA
 template <typename R>
 __device__ void recon_positivity(const Dev &d, const Par &p, int j, int lay, R *rec) {
   const int N = d.cs, NE = d.ne;
-  const R *xl = (const R *)d.exiL, *xr = (const R *)d.exiR;
+  const R *xs = (const R *)d.exi;
   R hmin = (R)INFINITY;
   for (int f = 0; f < 3; f++) {
     const int ce = d.cedge[f * N + j], e = ce >= 0 ? ce : ~ce;
-    const R *xs = ce >= 0 ? xl : xr;
+    const int o = ce >= 0 ? 0 : 2;
     for (int q = 0; q < 2; q++) {
-      const R x = xs[(2 * q) * NE + e], y = xs[(2 * q + 1) * NE + e];
+      const size_t at = ((size_t)q * NE + e) * 4 + o;
+      const R x = xs[at], y = xs[at + 1];
       R v[3];
       rec_values<R>(rec, x, y, v);
       const R h = ref_depth<R>(d, lay, e, q) + v[0];
@@ -502,7 +503,7 @@ template <typename R>
 __device__ __forceinline__ void own_write(const Dev &d, int e, int ell, int q, const R own[2], bool ok) {
   const R mine = q == 0 ? own[0] : own[1], theirs = q == 0 ? own[1] : own[0];
   const R m = (R)0.5 * (mine + __shfl_xor_sync(FULL, theirs, 1));
-  if (ok) ((R *)d.eO)[(2 * q + ell) * d.ne + e] = m;
+  if (ok) ((R *)d.eO)[((size_t)ell * d.ne + e) * 2 + q] = m;
 }
 
 // An edge's results for layer ell: the Gauss point q = 0 thread holds the
@@ -512,18 +513,16 @@ __device__ __forceinline__ void own_write(const Dev &d, int e, int ell, int q, c
 // W^n(x) (Eq. S2O3) and the interlayer source the cells' own levels.
 template <typename R>
 __device__ __forceinline__ void edge_write(const Dev &d, int e, int ell, int q, int stage, const R avg[6]) {
-  const int NE = d.ne;
-  const int vb = ell == 0 ? 3 : 0;
-  R *A = (R *)(q == 0 ? d.eF : d.eWn);
-  R *B = (R *)(q == 0 ? d.eFt : d.eWt);
-  const bool wa = q == 0 || stage == 1;
-  for (int k = 0; k < 3; k++) {
-    if (wa) A[(vb + k) * NE + e] = avg[k];
-    B[(vb + k) * NE + e] = avg[3 + k];
-  }
+  const size_t at = (size_t)ell * d.ne + e;
   if (q == 0) {
-    d.eFm[(vb / 3) * NE + e] = (double)avg[0];
-    d.eFtm[(vb / 3) * NE + e] = (double)avg[3];
+    const R f[4] = {avg[1], avg[2], avg[4], avg[5]};
+    const double m[2] = {(double)avg[0], (double)avg[3]};
+    store_n<R, 4>((R *)d.eF + 4 * at, f);
+    store_n<double, 2>(d.eM + 2 * at, m);
+  } else {
+    const R w[4] = {avg[0], avg[1], avg[2], 0}, wt[4] = {avg[3], avg[4], avg[5], 0};
+    if (stage == 1) store_n<R, 4>((R *)d.eWn + 4 * at, w);
+    store_n<R, 4>((R *)d.eWt + 4 * at, wt);
   }
 }
 
@@ -531,7 +530,7 @@ template <typename R>
 __device__ __forceinline__ void iface_body(const Dev &d) {
   int tid = blockIdx.x * blockDim.x + threadIdx.x;
   int e = tid >> 1, ell = tid & 1;
-  if (e >= d.ne || !running(d, d.inst[d.eL[e]])) return;
+  if (e >= d.ne || !running(d, d.eg[4 * (size_t)e + 3])) return;
   ((R *)d.hc)[ell * d.ne + e] = iface_any<R>(d, e, ell);
 }
 
@@ -545,7 +544,7 @@ __device__ __forceinline__ void edge_body(const Dev &d, const Par &p, int stage)
   // edges of instances still running are written
   R out[12], own[2];
   edge_any<R, false, true, POS>(d, p, ee, ell, q, stage, out, nullptr, own);
-  const bool ok = e < d.ne && running(d, d.inst[d.eL[ee]]);
+  const bool ok = e < d.ne && running(d, d.eg[4 * (size_t)ee + 3]);
   own_write<R>(d, e, ell, q, own, ok);
   // the Gauss point q = 0 thread averages the fluxes (out[0..5]), the q = 1
   // thread the interface values (out[6..11]): each sends the other its half
@@ -584,7 +583,7 @@ __device__ __forceinline__ void edge_fused_body(const Dev &d, const Par &p, int 
     const R mine = q == 0 ? out[k] : out[6 + k], theirs = q == 0 ? out[6 + k] : out[k];
     avg[k] = (R)0.5 * (mine + __shfl_xor_sync(FULL, theirs, 1));
   }
-  const bool ok = e < d.ne && running(d, d.inst[d.eL[ee]]);
+  const bool ok = e < d.ne && running(d, d.eg[4 * (size_t)ee + 3]);
   own_write<R>(d, e, ell, q, own, ok);
   // deferred units to the worklist, one atomic per warp
   const bool push = ok && q == 0 && !done;
@@ -826,7 +825,7 @@ template <typename R>
 __global__ void __launch_bounds__(128) k_init(Dev d, Par p, const int *perm, const double *grad_caller) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j < d.ne) {
-    const double R1 = d.ref[2 * d.inst[d.eL[j]] + 1];
+    const double R1 = d.ref[2 * d.eg[4 * (size_t)j + 3] + 1];
     ((R *)d.hrefe)[j] = (R)(R1 - d.eb0[j]);
     ((R *)d.hrefe)[d.ne + j] = (R)(R1 - d.eb1[j]);
   }
@@ -1014,25 +1013,20 @@ size_t layout(gks2l_ctx *c, char *base) {
   d.pos_flag = k.take<unsigned char>(2 * cs);
   d.pos_hbar = k.take<char>(rs * 2 * cs);
   d.wdev = k.take<float>(6 * cs);
-  d.eL = k.take<int>(ne);
-  d.eR = k.take<int>(ne);
-  d.exf = k.take<int8_t>(ne);
+  d.eg = k.take<int>(4 * ne);
   d.en = k.take<char>(rs * 2 * ne);
   d.eb0 = k.take<double>(ne);
   d.eb1 = k.take<double>(ne);
-  d.exiL = k.take<char>(rs * 4 * ne);
-  d.exiR = k.take<char>(rs * 4 * ne);
+  d.exi = k.take<char>(rs * 8 * ne);
   d.hrefe = k.take<char>(rs * 2 * ne);
   d.hc = k.take<char>(rs * 2 * ne);
   d.wl = k.take<int>(2 * ne);
   d.wl_count = k.take<int>(1);
-  d.eF = k.take<char>(rs * 6 * ne);
-  d.eFt = k.take<char>(rs * 6 * ne);
-  d.eFm = k.take<double>(2 * ne);
-  d.eFtm = k.take<double>(2 * ne);
+  d.eF = k.take<char>(rs * 8 * ne);
+  d.eM = k.take<double>(4 * ne);
   d.eO = k.take<char>(rs * 4 * ne);
-  d.eWt = k.take<char>(rs * 6 * ne);
-  d.eWn = k.take<char>(rs * 6 * ne);
+  d.eWt = k.take<char>(rs * 8 * ne);
+  d.eWn = k.take<char>(rs * 8 * ne);
   d.ref = k.take<double>(2 * ni);
   d.refR = k.take<char>(rs * 2 * ni);
   d.dt = k.take<double>(ni);
@@ -1491,7 +1485,22 @@ int gks2l_bind(gks2l_ctx *c, void *d_workspace, size_t bytes, void *stream) {
     ihs[j] = 1.0 / P.hs[j];
     epsA[j] = c->par.weno_eps * P.area[j];
   }
-  for (int e = 0; e < P.ne; e++) { en[e] = P.en0[e]; en[P.ne + e] = P.en1[e]; }
+  std::vector<int> eg(4 * (size_t)P.ne);
+  std::vector<double> exi(8 * (size_t)P.ne);
+  for (size_t e = 0; e < (size_t)P.ne; e++) {
+    en[2 * e] = P.en0[e];
+    en[2 * e + 1] = P.en1[e];
+    eg[4 * e] = P.eL[e];
+    eg[4 * e + 1] = P.eR[e];
+    eg[4 * e + 2] = P.exf[e];
+    eg[4 * e + 3] = P.inst[P.eL[e]];
+    for (size_t q = 0; q < 2; q++)
+      for (size_t k = 0; k < 2; k++) {
+        const size_t row = (2 * q + k) * P.ne + e, at = (q * P.ne + e) * 4 + k;
+        exi[at] = P.exiL[row];
+        exi[at + 2] = P.exiR[row];
+      }
+  }
   std::vector<double> xf(4 * kMaxXf, 0.0);
   std::copy(P.xf.begin(), P.xf.end(), xf.begin());
   int rc;
@@ -1501,14 +1510,14 @@ int gks2l_bind(gks2l_ctx *c, void *d_workspace, size_t bytes, void *stream) {
       (rc = upload_rows<int8_t>(c, c->d.st_xf, P.st_xf, kSlots)) || (rc = upload(c, c->d.tile_xf, txf)) ||
       (rc = upload_rows<int>(c, c->d.cedge, P.cedge, 3)) || (rc = upload_rows<double>(c, c->d.fsl, fsl, 3)) ||
       (rc = upload_form(c, c->d.fslR, fsl, 3, true)) ||
-      (rc = upload(c, c->d.inst_first, P.inst_first)) || (rc = upload(c, c->d.eL, P.eL)) ||
-      (rc = upload(c, c->d.eR, P.eR)) || (rc = upload(c, c->d.exf, P.exf)) || (rc = upload(c, c->d.xf, xf)) ||
+      (rc = upload(c, c->d.inst_first, P.inst_first)) || (rc = upload(c, c->d.eg, eg)) ||
+      (rc = upload(c, c->d.xf, xf)) ||
       (rc = upload(c, c->d_perm, P.perm)) ||
       (rc = c->rsize == 4 ? upload_tiles<float>(c) : upload_tiles<double>(c)) ||
       (rc = upload_form(c, c->d.plane, P.plane, 6, true)) ||
       (rc = upload_form(c, c->d.hsR, P.hs, 1, false)) || (rc = upload_form(c, c->d.ihsR, ihs, 1, false)) ||
-      (rc = upload_form(c, c->d.epsA, epsA, 1, false)) || (rc = upload_form(c, c->d.exiL, P.exiL, 1, false)) ||
-      (rc = upload_form(c, c->d.exiR, P.exiR, 1, false)) || (rc = upload_form(c, c->d.en, en, 1, false)))
+      (rc = upload_form(c, c->d.epsA, epsA, 1, false)) || (rc = upload_form(c, c->d.exi, exi, 1, false)) ||
+      (rc = upload_form(c, c->d.en, en, 1, false)))
     return rc;
   {
     std::vector<int> ch, ich(P.ninst + 1);
