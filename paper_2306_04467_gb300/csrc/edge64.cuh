@@ -7,7 +7,9 @@
 // a/b 8, sqrt 8, 1/x 5, rsqrt 5). The formulation here is the one with the
 // fewest (measured with 501 k triangles, 752 k edges): 1211 -> 777 per edge,
 // layer and point (k_edge<double> 6595 -> 4274 us) and 341 -> 274 per edge and
-// layer (k_iface<double> 954 -> 763 us):
+// layer (k_iface<double> 954 -> 763 us), then, with the sides' values kept by
+// k_iface and the results rotated once per edge, k_edge<double> 582 -> 496 us
+// at 65,522 triangles:
 //   - face-frame evaluation: the derivatives are formed along n and t at
 //     once, a mirrored side through the frame that its cell sees;
 //   - half-space moments split into a full-space and a boundary part, and the
@@ -38,9 +40,13 @@ struct ErfSeries {
     }
   }
 };
+// |x| <= 1/2 by the bits, off the FP64 pipe
+__host__ __device__ __forceinline__ bool within_half(double x) {
+  return (dbits(x) & 0x7fffffffffffffffll) <= 0x3fe0000000000000ll;
+}
 __host__ __device__ __forceinline__ double half_erf(double z) {
   constexpr ErfSeries S;
-  if (!(r_abs<double>(z) <= 0.5)) return 0.5 * erf(z);
+  if (!within_half(z)) return 0.5 * erf(z);
   const double y = D64::mul(z, z);
   double s = S.c[kErfTerms - 1];
 #pragma unroll
@@ -48,7 +54,7 @@ __host__ __device__ __forceinline__ double half_erf(double z) {
   return D64::mul(z, s);
 }
 __host__ __device__ __forceinline__ double half_erfc(double x) {
-  if (!(r_abs<double>(x) <= 0.5)) return 0.5 * erfc(x);
+  if (!within_half(x)) return 0.5 * erfc(x);
   return D64::sub(0.5, half_erf(x));
 }
 
@@ -107,30 +113,59 @@ __host__ __device__ __forceinline__ double blend64(double dl, double ul, double 
   return O::fma(half_erfc(O::mul(0.5, O::add(ul, ur))), O::sub(dl, dr), dr);
 }
 
-// iface_unit in the double form
-__host__ __device__ inline double iface_unit64(const Dev &d, int e, int ell) {
+// One side's values at a point: the level deviation, the velocity along n and
+// t and the depth's inverse root
+struct Point64 {
+  double d, U, V, r;
+};
+__host__ __device__ __forceinline__ Point64 point64(const double *w, const double m[10], const double fr[4],
+                                                    double href) {
+  using O = D64;
+  Point64 v;
+  v.d = poly_val64(w, m);
+  v.r = r_rsqrt(O::add(href, v.d));
+  const double ih = O::mul(v.r, v.r), mx = poly_val64(w + 12, m), my = poly_val64(w + 24, m);
+  v.U = O::mul(O::fma(mx, fr[0], O::mul(my, fr[1])), ih);
+  v.V = O::mul(O::fma(mx, fr[2], O::mul(my, fr[3])), ih);
+  return v;
+}
+
+// iface_unit in the double form, by two lanes, one per side (sd): each hands
+// the other its values at one point and blends at the other, and the two
+// layers' lanes form one point's monomials each and exchange. The sides' values
+// are kept for the edge solution (write), which would form them again.
+#ifdef __CUDACC__
+__device__ __forceinline__ double iface_unit64(const Dev &d, int e, int ell, int sd, bool write) {
   using O = D64;
   const EdgeIds g = edge_ids(d, e);
-  double x[2][4], n[2];
-  for (int q = 0; q < 2; q++) load_n<double, 4>((const double *)d.exi + ((size_t)q * d.ne + e) * 4, x[q]);
+  double x[2][2], n[2], fr[4], w[NREC], m[2][10], lev[2], un[2];
+  for (int q = 0; q < 2; q++) load_n<double, 2>((const double *)d.exi + ((size_t)q * d.ne + e) * 4 + 2 * sd, x[q]);
   load_n<double, 2>((const double *)d.en + 2 * (size_t)e, n);
-  const double n0 = n[0], n1 = n[1];
-  double lev[2][2], un[2][2];
-  for (int sd = 0; sd < 2; sd++) {
-    double fr[4], w[NREC];
-    face_frame(d, n0, n1, sd == 0 ? 0 : g.xf, fr);
-    load_rec<double, NREC>(d, ell, sd == 0 ? g.L : g.R, w);
-    for (int q = 0; q < 2; q++) {
-      double m[10];
-      monos64(x[q][2 * sd], x[q][2 * sd + 1], m);
-      lev[sd][q] = poly_val64(w, m);
-      const double r = r_rsqrt(O::add(ref_depth<double>(d, ell, e, q), lev[sd][q]));
-      un[sd][q] = O::mul(O::fma(poly_val64(w + 12, m), fr[0], O::mul(poly_val64(w + 24, m), fr[1])), O::mul(r, r));
+  face_frame(d, n[0], n[1], sd == 0 ? 0 : g.xf, fr);
+  load_rec<double, NREC>(d, ell, sd == 0 ? g.L : g.R, w);
+  {
+    double mine[10];
+    monos64(ell == 0 ? x[0][0] : x[1][0], ell == 0 ? x[0][1] : x[1][1], mine);
+    for (int k = 1; k < 10; k++) {
+      const double theirs = __shfl_xor_sync(0xffffffffu, mine[k], 2);
+      m[0][k] = ell == 0 ? mine[k] : theirs;
+      m[1][k] = ell == 0 ? theirs : mine[k];
     }
   }
-  return O::mul(0.5, O::add(blend64(lev[0][0], un[0][0], lev[1][0], un[1][0]),
-                            blend64(lev[0][1], un[0][1], lev[1][1], un[1][1])));
+  for (int q = 0; q < 2; q++) {
+    const Point64 v = point64(w, m[q], fr, ref_depth<double>(d, ell, e, q));
+    const double t[4] = {v.d, v.U, v.V, v.r};
+    if (write) store_n<double, 4>(d.ept + ((((size_t)e * 2 + ell) * 2 + q) * 2 + sd) * 4, t);
+    lev[q] = v.d;
+    un[q] = v.U;
+  }
+  const double ml = sd == 0 ? lev[0] : lev[1], mu = sd == 0 ? un[0] : un[1];
+  const double tl = __shfl_xor_sync(0xffffffffu, sd == 0 ? lev[1] : lev[0], 1);
+  const double tu = __shfl_xor_sync(0xffffffffu, sd == 0 ? un[1] : un[0], 1);
+  const double b = sd == 0 ? blend64(ml, mu, tl, tu) : blend64(tl, tu, ml, mu);
+  return O::mul(0.5, O::add(b, __shfl_xor_sync(0xffffffffu, b, 1)));
 }
+#endif
 
 // Edge-point side data for one layer, deviations, in the face's frame (n, t).
 struct Side64 {
@@ -156,10 +191,10 @@ __host__ __device__ __forceinline__ void level_dirs(const double *cf, const doub
 // of m, in the frame fr as that cell sees it; href is the depth of the
 // reference level at the point. OTHER: also the other layer's level
 // derivatives from its record (otherwise the caller takes them from the lane
-// that forms them as its own).
+// that forms them as its own). have: the side's values from k_iface, or null.
 template <bool OTHER>
 __host__ __device__ __forceinline__ void side64(const Dev &d, int ell, int c, int xf, const double fr[4],
-                                                const double m[10], double href, Side64 &s) {
+                                                const double m[10], double href, const double *have, Side64 &s) {
   using O = D64;
   double w[NREC];
   load_rec<double, NREC>(d, ell, c, w);
@@ -171,13 +206,20 @@ __host__ __device__ __forceinline__ void side64(const Dev &d, int ell, int c, in
     fs[2] = O::mul(fr[2], ih);
     fs[3] = O::mul(fr[3], ih);
   }
-  s.d = poly_val64(w, m);
-  s.h = O::add(href, s.d);
-  s.r = r_rsqrt(s.h);
-  s.ih = O::mul(s.r, s.r);
-  const double mx = poly_val64(w + 12, m), my = poly_val64(w + 24, m);
-  s.U = O::mul(O::fma(mx, fr[0], O::mul(my, fr[1])), s.ih);
-  s.V = O::mul(O::fma(mx, fr[2], O::mul(my, fr[3])), s.ih);
+  Point64 v;
+  if (have) {
+    double t[4];
+    load_n<double, 4>(have, t);
+    v = {t[0], t[1], t[2], t[3]};
+  } else {
+    v = point64(w, m, fr, href);
+  }
+  s.d = v.d;
+  s.h = O::add(href, v.d);
+  s.r = v.r;
+  s.ih = O::mul(v.r, v.r);
+  s.U = v.U;
+  s.V = v.V;
   level_dirs(w, m, fs, s.lev);
   // the depth is the level less the bottom in the lower layer (its slots 1, 2
   // carry grad B)
@@ -416,8 +458,9 @@ __host__ __device__ inline void gks_layer64(const Par &p, double href, const Sid
 // edge_unit in the double form (see there for the modes). The two lanes of an
 // edge's layer form one side's plane gradients each, and with PAIRED the two
 // layers' lanes one side's monomials each, and exchange: shuffles cost the
-// FP64 pipe nothing.
-template <bool FUSED, bool PAIRED, bool POS>
+// FP64 pipe nothing. HAVE: k_iface has left the sides' values. The vectors of
+// out stay in the face's frame.
+template <bool FUSED, bool PAIRED, bool POS, bool HAVE>
 __host__ __device__ inline bool edge_unit64(const Dev &d, const Par &p, int e, int ell, int q, double out[12],
                                             double *blend, double *own) {
   using O = D64;
@@ -456,8 +499,9 @@ __host__ __device__ inline bool edge_unit64(const Dev &d, const Par &p, int e, i
   }
 #endif
   Side64 s[2];
-  side64<!SH>(d, ell, cL, 0, fr[0], m[0], href, s[0]);
-  side64<!SH>(d, ell, cR, xf, fr[1], m[1], href, s[1]);
+  const double *have = HAVE ? d.ept + (((size_t)e * 2 + ell) * 2 + q) * 8 : nullptr;
+  side64<!SH>(d, ell, cL, 0, fr[0], m[0], href, have, s[0]);
+  side64<!SH>(d, ell, cR, xf, fr[1], m[1], href, HAVE ? have + 4 : nullptr, s[1]);
 #ifdef __CUDA_ARCH__
   if (SH) {
     for (int sd = 0; sd < 2; sd++)
@@ -520,14 +564,22 @@ __host__ __device__ inline bool edge_unit64(const Dev &d, const Par &p, int e, i
     own[1] = s[1].d;
   }
   if (FUSED && w < 1) return false;
-  double R[4][3];   // F, F_t, W, W_t
-  gks_layer64(p, href, s[0], s[1], D[0], D[1], dt, idt, R[0], R[1], R[2], R[3]);
-  for (int i = 0; i < 4; i++) {
-    out[3 * i] = R[i][0];
-    out[3 * i + 1] = O::fma(R[i][1], n0, -O::mul(R[i][2], n1));
-    out[3 * i + 2] = O::fma(R[i][1], n1, O::mul(R[i][2], n0));
-  }
+  gks_layer64(p, href, s[0], s[1], D[0], D[1], dt, idt, out, out + 3, out + 6, out + 9);   // F, F_t, W, W_t
   return true;
+}
+
+// The mean over an edge's two points of (F, F_t) or (W, W_t) from the points'
+// sum in the face's frame, in the global frame
+__host__ __device__ __forceinline__ void mean64(const Dev &d, int e, const double sum[6], double avg[6]) {
+  using O = D64;
+  double n[2];
+  load_n<double, 2>((const double *)d.en + 2 * (size_t)e, n);
+  const double h0 = O::mul(0.5, n[0]), h1 = O::mul(0.5, n[1]);
+  for (int k = 0; k < 6; k += 3) {
+    avg[k] = O::mul(0.5, sum[k]);
+    avg[k + 1] = O::fma(sum[k + 1], h0, -O::mul(sum[k + 2], h1));
+    avg[k + 2] = O::fma(sum[k + 1], h1, O::mul(sum[k + 2], h0));
+  }
 }
 
 }  // namespace gks2l

@@ -6,7 +6,7 @@
 //             compact P3/WENO reconstruction (Sec. 3.4); the tile's operator
 //             rows arrive in shared memory by bulk copy (cp.async.bulk)
 //             behind mbarriers
-//   k_iface   (edge x layer)         blended interface levels h-hat (Sec. 2.3)
+//   k_iface   (edge x layer; x side in FP64) blended interface levels h-hat (Sec. 2.3)
 //   k_edge    (edge x layer x point) gas-kinetic interface solution (Eq. SWE-2nd-order)
 //   k_update  (cell)                 fluxes, sources, S2O4 update, Gauss-theorem
 //                                    gradients (Eqs. SWE-semi-flux, slope-1, S2O3),
@@ -485,16 +485,30 @@ __global__ void k_harvest(Dev d, const int *perm, float tol, const float *logit_
   if (logits) logits[c] = logit_dev[j];
 }
 
-// the interface and edge units of a form
-template <typename R> __device__ __forceinline__ R iface_any(const Dev &d, int e, int ell) {
-  if constexpr (sizeof(R) == 8) return iface_unit64(d, e, ell);
-  else return iface_unit<R>(d, e, ell);
-}
-template <typename R, bool FUSED = false, bool PAIRED = false, bool POS = false>
+// the edge unit of a form
+template <typename R, bool FUSED = false, bool PAIRED = false, bool POS = false, bool HAVE = false>
 __device__ __forceinline__ bool edge_any(const Dev &d, const Par &p, int e, int ell, int q, int stage, R out[12],
                                          R *blend = nullptr, R *own = nullptr) {
-  if constexpr (sizeof(R) == 8) return edge_unit64<FUSED, PAIRED, POS>(d, p, e, ell, q, out, blend, own);
+  if constexpr (sizeof(R) == 8) return edge_unit64<FUSED, PAIRED, POS, HAVE>(d, p, e, ell, q, out, blend, own);
   else return edge_unit<R, FUSED, PAIRED, POS>(d, p, e, ell, q, stage, out, blend, own);
+}
+
+// The edge's results from its two points: the q = 0 thread takes the mean of
+// the fluxes (out[0..5]), the q = 1 thread that of the interface values
+// (out[6..11]); each sends the other its half.
+template <typename R>
+__device__ __forceinline__ void edge_mean(const Dev &d, int e, int q, const R out[12], R avg[6]) {
+  R sum[6];
+#pragma unroll
+  for (int k = 0; k < 6; k++) {
+    const R mine = q == 0 ? out[k] : out[6 + k], theirs = q == 0 ? out[6 + k] : out[k];
+    sum[k] = mine + __shfl_xor_sync(FULL, theirs, 1);
+  }
+  if constexpr (sizeof(R) == 8) {
+    mean64(d, e, sum, avg);
+  } else {
+    for (int k = 0; k < 6; k++) avg[k] = (R)0.5 * sum[k];
+  }
 }
 
 // Each side's own level of layer ell, the mean over the edge's two points:
@@ -529,9 +543,17 @@ __device__ __forceinline__ void edge_write(const Dev &d, int e, int ell, int q, 
 template <typename R>
 __device__ __forceinline__ void iface_body(const Dev &d) {
   int tid = blockIdx.x * blockDim.x + threadIdx.x;
-  int e = tid >> 1, ell = tid & 1;
-  if (e >= d.ne || !running(d, d.eg[4 * (size_t)e + 3])) return;
-  ((R *)d.hc)[ell * d.ne + e] = iface_any<R>(d, e, ell);
+  if constexpr (sizeof(R) == 8) {
+    // every thread computes (past the last edge: the last edge again): lanes
+    // of an edge exchange values
+    const int e = tid >> 2, ell = (tid >> 1) & 1, sd = tid & 1, ee = e < d.ne ? e : d.ne - 1;
+    const double v = iface_unit64(d, ee, ell, sd, e < d.ne);
+    if (sd == 0 && e < d.ne && running(d, d.eg[4 * (size_t)e + 3])) ((double *)d.hc)[(size_t)ell * d.ne + e] = v;
+  } else {
+    const int e = tid >> 1, ell = tid & 1;
+    if (e >= d.ne || !running(d, d.eg[4 * (size_t)e + 3])) return;
+    ((R *)d.hc)[(size_t)ell * d.ne + e] = iface_unit<R>(d, e, ell);
+  }
 }
 
 template <typename R, bool POS = false>
@@ -543,17 +565,11 @@ __device__ __forceinline__ void edge_body(const Dev &d, const Par &p, int stage)
   // its instance's dt is known, so the unit's loads issue at once; only
   // edges of instances still running are written
   R out[12], own[2];
-  edge_any<R, false, true, POS>(d, p, ee, ell, q, stage, out, nullptr, own);
+  edge_any<R, false, true, POS, true>(d, p, ee, ell, q, stage, out, nullptr, own);
   const bool ok = e < d.ne && running(d, d.eg[4 * (size_t)ee + 3]);
   own_write<R>(d, e, ell, q, own, ok);
-  // the Gauss point q = 0 thread averages the fluxes (out[0..5]), the q = 1
-  // thread the interface values (out[6..11]): each sends the other its half
   R avg[6];
-#pragma unroll
-  for (int k = 0; k < 6; k++) {
-    const R mine = q == 0 ? out[k] : out[6 + k], theirs = q == 0 ? out[6 + k] : out[k];
-    avg[k] = (R)0.5 * (mine + __shfl_xor_sync(FULL, theirs, 1));
-  }
+  edge_mean<R>(d, ee, q, out, avg);
   if (!ok) return;
   edge_write<R>(d, e, ell, q, stage, avg);
 }
@@ -578,11 +594,7 @@ __device__ __forceinline__ void edge_fused_body(const Dev &d, const Par &p, int 
   const R bo = __shfl_xor_sync(FULL, bl, 1);
   const R hcv = Rn<R>::mul((R)0.5, q == 0 ? Rn<R>::add(bl, bo) : Rn<R>::add(bo, bl));
   R avg[6];
-#pragma unroll
-  for (int k = 0; k < 6; k++) {
-    const R mine = q == 0 ? out[k] : out[6 + k], theirs = q == 0 ? out[6 + k] : out[k];
-    avg[k] = (R)0.5 * (mine + __shfl_xor_sync(FULL, theirs, 1));
-  }
+  edge_mean<R>(d, ee, q, out, avg);
   const bool ok = e < d.ne && running(d, d.eg[4 * (size_t)ee + 3]);
   own_write<R>(d, e, ell, q, own, ok);
   // deferred units to the worklist, one atomic per warp
@@ -618,11 +630,7 @@ __global__ void __launch_bounds__(128) k_edge_deferred(Dev d, Par p, int stage) 
     R out[12];
     edge_any<R>(d, p, e, ell, q, stage, out);
     R avg[6];
-#pragma unroll
-    for (int k = 0; k < 6; k++) {
-      const R mine = q == 0 ? out[k] : out[6 + k], theirs = q == 0 ? out[6 + k] : out[k];
-      avg[k] = (R)0.5 * (mine + __shfl_xor_sync(FULL, theirs, 1));
-    }
+    edge_mean<R>(d, e, q, out, avg);
     if (i >= n) continue;
     edge_write<R>(d, e, ell, q, stage, avg);
   }
@@ -1020,6 +1028,7 @@ size_t layout(gks2l_ctx *c, char *base) {
   d.exi = k.take<char>(rs * 8 * ne);
   d.hrefe = k.take<char>(rs * 2 * ne);
   d.hc = k.take<char>(rs * 2 * ne);
+  d.ept = k.take<double>(rs == 8 ? 32 * ne : 0);
   d.wl = k.take<int>(2 * ne);
   d.wl_count = k.take<int>(1);
   d.eF = k.take<char>(rs * 8 * ne);
@@ -1219,7 +1228,7 @@ template <typename R> bool spread(const gks2l_ctx *c, size_t n) {
 
 template <typename R>
 void launch_iface(gks2l_ctx *c, cudaStream_t st) {
-  const size_t n = 2 * (size_t)c->d.ne;
+  const size_t n = (sizeof(R) == 8 ? 4 : 2) * (size_t)c->d.ne;
   GKS2L_SHAPE_SWITCH(c->shape[0], k_iface, n, st, c->d)
 }
 
