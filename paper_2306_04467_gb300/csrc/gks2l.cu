@@ -192,6 +192,7 @@ __global__ void __launch_bounds__(TW * 6 / ReconCfg<R>::VP, ReconCfg<R>::BLOCKS)
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(T::TX_LINEAR)
                  : "memory");
     bulk_load(sm, src, T::TX_LINEAR, bar);
+    if (blockIdx.x == 0 && blockIdx.y == 0) *d.wl_count = 0;   // for the fused edge kernel that follows
     if (!T::REUSE && !all_linear) {
       asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar2)), "r"(T::TX2)
                    : "memory");
@@ -303,7 +304,10 @@ __global__ void __launch_bounds__(TW * 6 / ReconCfg<R>::VP, ReconCfg<R>::BLOCKS)
 // tiles of 32 cells: the 24 features of each cell go to a shared-memory tile,
 // the network runs on the tensor cores, and the warp writes the tile's mask
 // (cells past the end or of finished instances count as smooth).
-constexpr int GATE_BLOCKS_PER_SM = 2;
+// k_gate: as many as its registers allow, latency-bound warps (alone 26.5 ->
+// 18.0 us at 181 k triangles against two per SM)
+constexpr int GATE_BLOCKS_PER_SM = 5;
+constexpr int GATE_TC_BLOCKS_PER_SM = 2;   // k_gate_tc, times the variant's factor
 
 template <typename R>
 __global__ void __launch_bounds__(128) k_gate(Dev d, Par p) {
@@ -1178,7 +1182,8 @@ inline bool gate_plain_edges(int v) { return v >= 2 * kGateKernels; }
 template <typename R>
 void launch_gate(gks2l_ctx *c, const Par &p, cudaStream_t st) {
   const int kernel = gate_kernel(c->shape[3]);
-  const unsigned per_sm = GATE_BLOCKS_PER_SM * (kernel == 3 ? 4 : kernel == 2 ? 2 : 1);
+  const unsigned per_sm =
+      kernel == 0 ? GATE_BLOCKS_PER_SM : GATE_TC_BLOCKS_PER_SM * (kernel == 3 ? 4 : kernel == 2 ? 2 : 1);
   const unsigned nb = std::min(blocks(c->d.nt, 4 * TW), (unsigned)(c->n_sm * per_sm));
   if (kernel >= 1) k_gate_tc<R><<<nb, GATE_TC_M, 0, st>>>(c->d, p);
   else k_gate<R><<<nb, 128, 0, st>>>(c->d, p);
@@ -1243,11 +1248,11 @@ void launch_edge(gks2l_ctx *c, const Par &p, int stage, cudaStream_t st) {
   GKS2L_SHAPE_SWITCH(c->shape[1], k_edge, n, st, c->d, p, stage)
 }
 
-// gated runs: interface levels and edge solution fused, then the deferred units
+// gated runs: interface levels and edge solution fused, then the deferred
+// units (the reconstruction has cleared their count)
 template <typename R>
 void launch_edge_fused(gks2l_ctx *c, const Par &p, int stage, cudaStream_t st) {
   const size_t n = 4 * (size_t)c->d.ne;
-  cudaMemsetAsync(c->d.wl_count, 0, sizeof(int), st);
   GKS2L_SHAPE_SWITCH(c->shape[1], k_edgef, n, st, c->d, p, stage)
 }
 template <typename R>
