@@ -691,23 +691,20 @@ __global__ void k_mass(Dev d) {
   }
 }
 
-template <typename R>
+template <typename R, int NL = 2>
 __device__ __forceinline__ void update_body(const Dev &d, const Par &p, int stage) {
-  int j = blockIdx.x * blockDim.x + threadIdx.x;
-  bool ok = j < d.nt;
-  int inst = ok ? d.inst[j] : 0;
-  double ratio = INFINITY;
+  const int tid = blockIdx.x * blockDim.x + threadIdx.x;
+  const int j = NL == 2 ? tid : tid >> 1, lay = NL == 2 ? 0 : tid & 1, jj = j < d.nt ? j : d.nt - 1;
+  const bool ok = j < d.nt;
+  const int inst = d.inst[jj];
   int fl = 0;
-  if (ok) {
-    double r = update_unit<R>(d, p, j, stage, &fl);
-    if (r > 0) ratio = r;
-  }
+  const double r = update_unit<R, NL>(d, p, jj, lay, stage, ok, &fl);
   if (fl) atomicOr(d.status, fl);
   // the gate has joined: its mask becomes the next reconstruction's
-  if (p.use_gate && ok && (j & (TW - 1)) == 0) d.gate_mask[j / TW] = d.gate_next[j / TW];
+  if (p.use_gate && ok && lay == 0 && (j & (TW - 1)) == 0) d.gate_mask[j / TW] = d.gate_next[j / TW];
   if (stage != 2) return;
-  reduce_cfl(d, ok, inst, ratio);
-  if (ok && j == d.inst_first[inst]) d.t[inst] += d.dt[inst];
+  reduce_cfl(d, ok, inst, dbits(r) > 0 ? r : INFINITY);
+  if (ok && lay == 0 && j == d.inst_first[inst]) d.t[inst] += d.dt[inst];
 }
 
 // The interface, edge (fused edge) and update kernels come in five launch
@@ -716,14 +713,27 @@ __device__ __forceinline__ void update_body(const Dev &d, const Par &p, int stag
 // the entry points differ in their launch bounds only.
 template <typename R, int BS>
 __global__ void __launch_bounds__(BS) k_iface(Dev d) { iface_body<R>(d); }
+// (the edge kernel in FP32 with 96 registers, ten blocks of 64 per SM: 283 us at
+// 1.04 M triangles; left alone it takes 80 and 321 us)
 template <typename R, int BS>
-__global__ void __launch_bounds__(BS) k_edge(Dev d, Par p, int stage) { edge_body<R>(d, p, stage); }
-// (the fused kernel's default shapes are held in FP32 to 768 resident threads
-// per SM, the 80 registers its body compiles to when left alone)
+__global__ void __launch_bounds__(BS, sizeof(R) == 4 && BS > 32 ? 640 / BS : 1) k_edge(Dev d, Par p, int stage) {
+  edge_body<R>(d, p, stage);
+}
+// (the fused kernel in FP32 with 72 registers, thirteen blocks of 64 per SM:
+// 282 us at 1.04 M triangles against 288 with the 80 that it takes when left
+// alone)
 template <typename R, int BS>
-__global__ void __launch_bounds__(BS, sizeof(R) == 4 && BS > 32 ? 768 / BS : 1) k_edgef(Dev d, Par p, int stage) { edge_fused_body<R>(d, p, stage); }
+__global__ void __launch_bounds__(BS, sizeof(R) == 4 && BS > 32 ? 832 / BS : 1) k_edgef(Dev d, Par p, int stage) { edge_fused_body<R>(d, p, stage); }
+// (the update waits for its gathers: held in FP32 to 896 resident threads per
+// SM, 72 registers, 130 us at 1.04 M triangles against 152 with the 92 that it
+// takes when left alone)
 template <typename R, int BS>
-__global__ void __launch_bounds__(BS) k_update(Dev d, Par p, int stage) { update_body<R>(d, p, stage); }
+__global__ void __launch_bounds__(BS, (sizeof(R) == 4 ? 896 : 512) / BS) k_update(Dev d, Par p, int stage) {
+  update_body<R>(d, p, stage);
+}
+// the update of a small mesh, a layer per thread
+template <typename R, int BS>
+__global__ void __launch_bounds__(BS) k_update_layer(Dev d, Par p, int stage) { update_body<R, 1>(d, p, stage); }
 // the edge solution with the positivity option (one launch shape)
 template <typename R, int BS>
 __global__ void __launch_bounds__(BS) k_edge_pos(Dev d, Par p, int stage) { edge_body<R, true>(d, p, stage); }
@@ -873,7 +883,8 @@ __global__ void __launch_bounds__(128) k_init(Dev d, Par p, const int *perm, con
     if (!p.use_gate && j % TW == 0) d.gate_mask[j / TW] = 0u;
     if (!fl && (w[0] <= 0 || w[3] <= 0)) fl = 1;
     if (!fl) {
-      ratio = cfl_ratio<R>(w, d.dX[j], pv<R>(p.g, p.gf));
+      const R G = pv<R>(p.g, p.gf);
+      ratio = cfl_ratio<R>(layer_speed<R>(w[0], w[1], w[2], G), layer_speed<R>(w[3], w[4], w[5], G), d.dX[j]);
       if (!(ratio > 0) || !isfinite(ratio)) fl = 2;
     }
     if (fl) {
@@ -963,7 +974,7 @@ struct gks2l_ctx {
   bool has_mlp = false;
   int n_sm = 1;                // SMs of the bound device
   cudaStream_t side = nullptr; // second stream for the gate (created with the network)
-  int shape[4] = {1, 1, 1, 0}; // launch shapes of the interface, edge and update kernels; gate variant
+  int shape[4] = {0, 0, 1, 0}; // launch shapes of the interface, edge and update kernels; gate variant
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   int phase = 0;
   int64_t stages = 0;
@@ -1263,6 +1274,16 @@ void launch_edge_deferred(gks2l_ctx *c, const Par &p, int stage, cudaStream_t st
 template <typename R>
 void launch_update(gks2l_ctx *c, const Par &p, int stage, cudaStream_t st) {
   const size_t n = (size_t)c->d.nt;
+  // A mesh that does not fill the SMs' threads is bound by the length of one
+  // thread's chain of loads (and in FP64 of its FP64 operations): a layer per
+  // thread, 10.2 -> 8.2 us at 4,608 triangles, 15.3 -> 13.1 at 512 in FP64; at
+  // 181 k and beyond both layers per thread are as fast or faster (130 against
+  // 139 us at 1.04 M), in FP64 from 66 k on (41 against 46 us).
+  if (c->shape[2] < 3 && blocks(n, 128) < 2 * (unsigned)c->n_sm) {
+    if (spread<R>(c, 2 * n)) k_update_layer<R, 32><<<blocks(2 * n, 32), 32, 0, st>>>(c->d, p, stage);
+    else k_update_layer<R, 128><<<blocks(2 * n, 128), 128, 0, st>>>(c->d, p, stage);
+    return;
+  }
   GKS2L_SHAPE_SWITCH(c->shape[2], k_update, n, st, c->d, p, stage)
 }
 
@@ -1404,10 +1425,17 @@ int after_state(gks2l_ctx *c, const double *grad_caller) {
   return 0;
 }
 
+// the context's arrays with avg the current state (W* between a step's stages)
+Dev current(const gks2l_ctx *c) {
+  Dev d = c->d;
+  if (c->phase == 1) d.avg = d.Wn;
+  return d;
+}
+
 void launch_read(gks2l_ctx *c, double *avg, double *grad) {
   const unsigned nb = blocks(c->d.nt, 128);
-  if (c->par.precision == GKS2L_FP32) k_read<float><<<nb, 128, 0, c->stream>>>(c->d, c->d_perm, avg, grad);
-  else k_read<double><<<nb, 128, 0, c->stream>>>(c->d, c->d_perm, avg, grad);
+  if (c->par.precision == GKS2L_FP32) k_read<float><<<nb, 128, 0, c->stream>>>(current(c), c->d_perm, avg, grad);
+  else k_read<double><<<nb, 128, 0, c->stream>>>(current(c), c->d_perm, avg, grad);
 }
 
 int create_impl(int n, const gks2l_mesh *meshes, const gks2l_params *params, gks2l_ctx **out) {
@@ -1777,7 +1805,7 @@ int gks2l_stats(gks2l_ctx *c, gks2l_stats_t *out) {
   int st = 0;
   unsigned long long cnt[2] = {0, 0};
   CK(cudaMemsetAsync(c->d.mass, 0, mass.size() * sizeof(double), c->stream));
-  k_mass<<<blocks(c->prep.nt, 128), 128, 0, c->stream>>>(c->d);
+  k_mass<<<blocks(c->prep.nt, 128), 128, 0, c->stream>>>(current(c));
   CK(cudaGetLastError());
   CK(cudaMemcpyAsync(mass.data(), c->d.mass, mass.size() * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   CK(cudaMemcpyAsync(&t, c->d.t, sizeof(double), cudaMemcpyDeviceToHost, c->stream));

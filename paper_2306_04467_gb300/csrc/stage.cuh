@@ -77,7 +77,8 @@ struct Dev {
   double *avg;              // state averages [v][cell] (FP64)
   void *dq, *dg;            // deviation mirrors [pair][cell][2] and gradients [pair][cell][2][2], type R
   void *hrefc;              // R1 - B_j per cell, type R
-  double *Wn, *Ln, *Ltn;    // stage snapshot (FP64; L and L_t rows of the layer depths only)
+  double *Wn, *Ln, *Ltn;    // W* between a step's stages (avg keeps W^n), and the stage-1 L and
+                            // L_t (rows of the layer depths only), FP64
   void *incR;               // [4][cell] stage-1 part of the stage-2 momentum increment, type R
   void *srec;               // side records [tile][layer][vector][32][16 bytes], type R (lower layer first)
   void *omg;                // omega_H / gamma_H of eta1 [0] and h2 [1], type R
@@ -1209,45 +1210,54 @@ __host__ __device__ inline bool edge_unit(const Dev &d, const Par &p, int e, int
 }
 
 // ------------------------------------------------------------- cell unit
-// dX / U_max of a cell state w (Sec. 4: U_max the larger over the layers of
-// |U| + sqrt(G h)) in the form's precision; the update kernel and the kernel
-// that starts a newly set state both use it, so a restarted run takes the
-// same steps as an uninterrupted one. FP32 form: the reciprocal in single
-// precision (dt to ~1e-7 relative), sparing the FP64 pipe a double division.
+// dX / U_max of a cell (Sec. 4: U_max the larger over the layers of |U| +
+// sqrt(G h)) in the form's precision; the update kernel and the kernel that
+// starts a newly set state both use it, so a restarted run takes the same
+// steps as an uninterrupted one. FP32 form: the reciprocal in single precision
+// (dt to ~1e-7 relative), sparing the FP64 pipe a double division.
 template <typename R>
-__host__ __device__ inline double cfl_ratio(const double w[NV], double dX, R G) {
+__host__ __device__ inline R layer_speed(double h_, double mx, double my, R G) {
+  R h = (R)h_, u = (R)mx / h, v = (R)my / h;
+  return r_sqrt<R>(u * u + v * v) + r_sqrt<R>(G * h);
+}
+template <typename R>
+__host__ __device__ inline double cfl_ratio(R upper, R lower, double dX) {
   R um = 0;
-  for (int l = 0; l < 2; l++) {
-    R h = (R)w[3 * l], u = (R)w[3 * l + 1] / h, v = (R)w[3 * l + 2] / h;
-    R sp = r_sqrt<R>(u * u + v * v) + r_sqrt<R>(G * h);
-    um = sp > um ? sp : um;
-  }
+  um = upper > um ? upper : um;
+  um = lower > um ? lower : um;
   if (sizeof(R) == 4) return dX * (double)((R)1 / um);
   return dX / (double)um;
 }
 
+#ifdef __CUDACC__
 // Flux and source residuals, S2O4 update (Eq. SWE-fully-discrete), interface
-// values at the stage end (Eq. S2O3) and Gauss-theorem gradients (Eq. slope-1).
-// Returns the CFL ratio dX/U_max of the new state (stage 2) or 0.
-template <typename R>
-__host__ __device__ inline double update_unit(const Dev &d, const Par &p, int j, int stage, int *flags) {
+// values at the stage end (Eq. S2O3) and Gauss-theorem gradients (Eq. slope-1)
+// of a cell: of both its layers (NL = 2), or of one (NL = 1, lay: 0 lower, 1
+// upper) with the other layer in the next or previous lane, the two exchanging
+// what each needs of the other. All lanes of the warp call; only with `ok` are
+// results written. Returns the CFL ratio dX/U_max of the new state (stage 2)
+// or 0. Between the stages of a step d.avg keeps W^n and d.Wn holds W*.
+template <typename R, int NL>
+__device__ __forceinline__ double update_unit(const Dev &d, const Par &p, int j, int lay, int stage, bool ok,
+                                              int *flags) {
   const int N = d.cs;
   const size_t NE = (size_t)d.ne;
   const int in = d.inst[j];
   const double dt = d.dt[in];
   // the unit's loads and arithmetic do not wait on dt: a cell of an instance
   // that has stopped (dt = 0) is computed too, and only its writes are dropped
-  const bool act = dt > 0;
+  const bool act = ok && dbits(dt) > 0;
   const R dtr = ((const R *)d.dtR)[in];
   const R cend = stage == 1 ? (R)0.5 * dtr : dtr;
-  // mass residuals in FP64 (exact conservation), the rest in R
-  double LFm[2] = {0, 0}, LFtm[2] = {0, 0};
-  R LF[NV] = {0}, LFt[NV] = {0}, mWt[NV] = {0};
-  R GGt[NV][2] = {{0}}, GGn[NV][2] = {{0}};
-  // the interlayer source's point values (R16): this cell's own levels at its
-  // six Gauss points, their mean (mO) and Gauss-theorem gradient (GO), for
-  // the lower (0: eta1 - R1) and upper (1: h2 - R2) layer
-  R mO[2] = {0, 0}, GO[2][2] = {{0, 0}, {0, 0}};
+  // by layer (i = 0 .. NL - 1, or the one of the lane): mass residuals in FP64
+  // (exact conservation), the rest in R; LF, LFt: the discharge's; mWt, GGt:
+  // mean and Gauss-theorem gradient of the depth's W_t; GGn: gradients at the
+  // stage end; the interlayer source's point values (R16), this cell's own
+  // levels at its six Gauss points: their mean (mO) and Gauss-theorem gradient
+  // (GO)
+  double LFm[NL] = {}, LFtm[NL] = {};
+  R LF[NL][2] = {}, LFt[NL][2] = {}, mWt[NL] = {}, GGt[NL][2] = {}, GGn[NL][3][2] = {}, mO[NL] = {}, GO[NL][2] = {};
+#pragma unroll
   for (int f = 0; f < 3; f++) {
     int ce = d.cedge[f * N + j];
     int e = ce >= 0 ? ce : ~ce;
@@ -1257,8 +1267,9 @@ __host__ __device__ inline double update_unit(const Dev &d, const Par &p, int j,
     R n[2];
     load_n<R, 2>((const R *)d.en + 2 * (size_t)e, n);
     const R snx = slR * n[0], sny = slR * n[1];
-    for (int l = 0; l < 2; l++) {
-      const size_t at = l * NE + e;
+#pragma unroll
+    for (int i = 0; i < NL; i++) {
+      const size_t at = (NL == 2 ? i : lay) * NE + e;
       R F[4], Wt[4], Wn[4];
       double M[2];
       load_n<R, 4>((const R *)d.eF + 4 * at, F);
@@ -1266,102 +1277,122 @@ __host__ __device__ inline double update_unit(const Dev &d, const Par &p, int j,
       load_n<R, 4>((const R *)d.eWn + 4 * at, Wn);
       load_n<double, 2>(d.eM + 2 * at, M);
       const R o = ((const R *)d.eO)[2 * at + side];
-      const int v0 = l == 0 ? 3 : 0;                 // the layer's depth variable
-      mO[l] += o * (R)(1.0 / 3.0);
-      GO[l][0] += snx * o; GO[l][1] += sny * o;
-      LFm[v0 / 3] -= sl * M[0];
-      LFtm[v0 / 3] -= sl * M[1];
-      mWt[v0] += Wt[0] * (R)(1.0 / 3.0);
-      GGt[v0][0] += snx * Wt[0]; GGt[v0][1] += sny * Wt[0];
-      for (int i = 0; i < 2; i++) {
-        LF[v0 + 1 + i] -= slR * F[i];
-        LFt[v0 + 1 + i] -= slR * F[2 + i];
+      mO[i] += o * (R)(1.0 / 3.0);
+      GO[i][0] += snx * o; GO[i][1] += sny * o;
+      LFm[i] -= sl * M[0];
+      LFtm[i] -= sl * M[1];
+      mWt[i] += Wt[0] * (R)(1.0 / 3.0);
+      GGt[i][0] += snx * Wt[0]; GGt[i][1] += sny * Wt[0];
+      for (int k = 0; k < 2; k++) {
+        LF[i][k] -= slR * F[k];
+        LFt[i][k] -= slR * F[2 + k];
       }
-      for (int i = 0; i < 3; i++) {
-        R We = Wn[i] + cend * Wt[i];
-        GGn[v0 + i][0] += snx * We; GGn[v0 + i][1] += sny * We;
+      for (int k = 0; k < 3; k++) {
+        R We = Wn[k] + cend * Wt[k];
+        GGn[i][k][0] += snx * We; GGn[i][k][1] += sny * We;
       }
     }
   }
+  R GOo[NL][2], GGto[NL][2];                       // the other layer's
+  for (int i = 0; i < NL; i++)
+    for (int k = 0; k < 2; k++) {
+      GOo[i][k] = NL == 2 ? GO[NL - 1 - i][k] : __shfl_xor_sync(0xffffffffu, GO[i][k], 1);
+      GGto[i][k] = NL == 2 ? GGt[NL - 1 - i][k] : __shfl_xor_sync(0xffffffffu, GGt[i][k], 1);
+    }
   const R G = pv<R>(p.g, p.gf), chi = pv<R>(p.chi, p.chif);
-  R gb[2], dq0[2];   // the levels' deviations (h2, eta1)
+  R gb[2], dq0[2], speed[NL], q0[NL], g0[NL][2];   // dq0: the levels' deviations (h2, eta1)
   load_n<R, 2>((const R *)d.bgR + 2 * (size_t)j, gb);
   load_n<R, 2>(dq_at<R>(d, 0, j), dq0);
-  const R R2 = ((const R *)d.refR)[2 * in];
-  const R hrc = ((const R *)d.hrefc)[j];          // R1 - B_j
-  const R m1 = hrc + mO[0], m2 = R2 + mO[1];       // means of h1, h2 over the 6 Gauss points
-  const R LFh2 = (R)LFm[0], LFh1 = (R)LFm[1];
-  R L[NV], Lt[NV];
-  for (int k = 0; k < 2; k++) {
-    // upper layer: -G h2 grad(B + h1) with h1 = eta1 - B at the points; the
-    // time derivative by the product rule with the interface solution's W_t (R4)
-    L[1 + k] = LF[1 + k] - G * (dq0[0] - mO[1]) * gb[k] - G * m2 * GO[0][k];
-    Lt[1 + k] = LFt[1 + k] - G * (LFh2 - mWt[0]) * gb[k] - G * mWt[0] * GO[0][k] - G * m2 * GGt[3][k];
-    // lower layer: flux reference pressure + bottom source -> -G (eta1 - R1) grad B; interlayer -chi G h1 grad h2
-    L[4 + k] = LF[4 + k] - G * dq0[1] * gb[k] - chi * G * m1 * GO[1][k];
-    Lt[4 + k] = LFt[4 + k] - G * LFh1 * gb[k] - chi * G * (mWt[3] * GO[1][k] + m1 * GGt[0][k]);
-  }
-  // S2O4 (Eq. SWE-fully-discrete): stage 1 W* = W^n + dt/2 L^n + dt^2/8 L_t^n;
-  // stage 2 W^{n+1} = W^n + dt L^n + dt^2/6 L_t^n + dt^2/3 L_t^*. The layer
-  // depths (exact conservation) in FP64 throughout; the momenta's increments
-  // in R (their residuals are R), each added to the FP64 state once
-  const int mom[4] = {1, 2, 4, 5};
-  double nw[NV];
-  for (int m = 0; m < 2; m++) {
-    const int v = 3 * m;
-    const double a = d.avg[v * N + j];
-    if (stage == 1) {
-      if (act) {
-        d.Wn[v * N + j] = a;
-        d.Ln[v * N + j] = LFm[m];
-        d.Ltn[v * N + j] = LFtm[m];
-      }
-      nw[v] = a + 0.5 * dt * LFm[m] + 0.125 * dt * dt * LFtm[m];
-    } else {
-      nw[v] = d.Wn[v * N + j] + dt * d.Ln[v * N + j] + dt * dt * (1.0 / 6.0) * d.Ltn[v * N + j] +
-              dt * dt * (1.0 / 3.0) * LFtm[m];
-    }
-  }
-  R *inc = (R *)d.incR;
   const R dt2 = dtr * dtr;
-  for (int i = 0; i < 4; i++) {
-    const int v = mom[i];
-    const double a = d.avg[v * N + j];
+  int fl = 0;
+#pragma unroll
+  for (int i = 0; i < NL; i++) {
+    const int l = NL == 2 ? i : lay, v0 = l == 0 ? 3 : 0;   // the layer and its depth variable
+    const R LFh = (R)LFm[i];
+    R L[2], Lt[2];
+    if (l == 1) {
+      // upper layer: -G h2 grad(B + h1) with h1 = eta1 - B at the points; the
+      // time derivative by the product rule with the interface solution's W_t (R4)
+      const R m2 = ((const R *)d.refR)[2 * in] + mO[i];   // mean of h2 over the 6 Gauss points
+      for (int k = 0; k < 2; k++) {
+        L[k] = LF[i][k] - G * (dq0[0] - mO[i]) * gb[k] - G * m2 * GOo[i][k];
+        Lt[k] = LFt[i][k] - G * (LFh - mWt[i]) * gb[k] - G * mWt[i] * GOo[i][k] - G * m2 * GGto[i][k];
+      }
+    } else {
+      // lower layer: flux reference pressure + bottom source -> -G (eta1 - R1) grad B; interlayer -chi G h1 grad h2
+      const R m1 = ((const R *)d.hrefc)[j] + mO[i];       // (R1 - B_j) + the mean level's deviation
+      for (int k = 0; k < 2; k++) {
+        L[k] = LF[i][k] - G * dq0[1] * gb[k] - chi * G * m1 * GOo[i][k];
+        Lt[k] = LFt[i][k] - G * LFh * gb[k] - chi * G * (mWt[i] * GOo[i][k] + m1 * GGto[i][k]);
+      }
+    }
+    // S2O4 (Eq. SWE-fully-discrete): stage 1 W* = W^n + dt/2 L^n + dt^2/8 L_t^n;
+    // stage 2 W^{n+1} = W^n + dt L^n + dt^2/6 L_t^n + dt^2/3 L_t^*. The layer
+    // depths (exact conservation) in FP64 throughout; the momenta's increments
+    // in R (their residuals are R), each added to the FP64 state once
+    double nw[3], was[3];
+    double *now = (stage == 1 ? d.Wn : d.avg) + (size_t)v0 * N + j;
+    double *Ln = d.Ln + (size_t)v0 * N + j, *Ltn = d.Ltn + (size_t)v0 * N + j;
+    R *inc = (R *)d.incR + (size_t)(l == 1 ? 0 : 2) * N + j;
+    for (int k = 0; k < 3; k++) was[k] = d.avg[(size_t)(v0 + k) * N + j];
     if (stage == 1) {
       if (act) {
-        d.Wn[v * N + j] = a;
-        inc[i * N + j] = dtr * L[v] + dt2 * (R)(1.0 / 6.0) * Lt[v];
+        *Ln = LFm[i];
+        *Ltn = LFtm[i];
       }
-      nw[v] = a + (double)((R)0.5 * dtr * L[v] + (R)0.125 * dt2 * Lt[v]);
+      nw[0] = was[0] + 0.5 * dt * LFm[i] + 0.125 * dt * dt * LFtm[i];
     } else {
-      nw[v] = d.Wn[v * N + j] + (double)(inc[i * N + j] + dt2 * (R)(1.0 / 3.0) * Lt[v]);
+      nw[0] = was[0] + dt * *Ln + dt * dt * (1.0 / 6.0) * *Ltn + dt * dt * (1.0 / 3.0) * LFtm[i];
     }
+    for (int k = 0; k < 2; k++) {
+      if (stage == 1) {
+        if (act) inc[(size_t)k * N] = dtr * L[k] + dt2 * (R)(1.0 / 6.0) * Lt[k];
+        nw[1 + k] = was[1 + k] + (double)((R)0.5 * dtr * L[k] + (R)0.125 * dt2 * Lt[k]);
+      } else {
+        nw[1 + k] = was[1 + k] + (double)(inc[(size_t)k * N] + dt2 * (R)(1.0 / 3.0) * Lt[k]);
+      }
+    }
+    // (W* of a cell that has stopped is its state: the one read between stages)
+    if (act || (ok && stage == 1))
+      for (int k = 0; k < 3; k++) now[(size_t)k * N] = act ? nw[k] : was[k];
+    // the level's deviation and gradient (of the lower layer: grad h1 = grad
+    // eta1 - grad B, the interface values being water levels)
+    const double lev = l == 0 ? nw[0] + d.bmean[j] : nw[0];
+    q0[i] = (R)(lev - d.ref[2 * in + 1 - l]);
+    for (int k = 0; k < 2; k++) g0[i][k] = l == 0 ? GGn[i][0][k] - gb[k] : GGn[i][0][k];
+    if (act) {
+      const int pair = l == 1 ? 1 : 2;
+      const R q[2] = {(R)nw[1], (R)nw[2]}, g[4] = {GGn[i][1][0], GGn[i][1][1], GGn[i][2][0], GGn[i][2][1]};
+      store_n<R, 2>(dq_at<R>(d, pair, j), q);
+      store_n<R, 4>(dg_at<R>(d, pair, j), g);
+    }
+    // health flags by integer tests on the bits (off the FP64 pipe)
+    for (int k = 0; k < 3; k++)
+      if (!finite_bits(nw[k]) || !isfinite(GGn[i][k][0]) || !isfinite(GGn[i][k][1])) fl |= 2;
+    if (!(dbits(nw[0]) > 0)) fl |= 1;
+    if (stage == 2) speed[i] = layer_speed<R>(nw[0], nw[1], nw[2], G);
   }
   if (act) {
-    for (int v = 0; v < NV; v++) d.avg[v * N + j] = nw[v];
-    const R q[NPAIR][2] = {{(R)(nw[0] - d.ref[2 * in]), (R)((nw[3] + d.bmean[j]) - d.ref[2 * in + 1])},
-                           {(R)nw[1], (R)nw[2]},
-                           {(R)nw[4], (R)nw[5]}};
-    for (int i = 0; i < NPAIR; i++) {
-      const int v0 = var_of(i, 0), v1 = var_of(i, 1);
-      R g[4] = {GGn[v0][0], GGn[v0][1], GGn[v1][0], GGn[v1][1]};
-      if (i == 0) {
-        // the interface values of variable 3 are water levels: grad h1 = grad eta1 - grad B
-        g[2] -= gb[0];
-        g[3] -= gb[1];
-      }
-      store_n<R, 2>(dq_at<R>(d, i, j), q[i]);
-      store_n<R, 4>(dg_at<R>(d, i, j), g);
+    if (NL == 2) {
+      const R q[2] = {q0[NL - 1], q0[0]}, g[4] = {g0[NL - 1][0], g0[NL - 1][1], g0[0][0], g0[0][1]};
+      store_n<R, 2>(dq_at<R>(d, 0, j), q);
+      store_n<R, 4>(dg_at<R>(d, 0, j), g);
+    } else {
+      dq_at<R>(d, 0, j)[1 - lay] = q0[0];
+      store_n<R, 2>(dg_at<R>(d, 0, j) + 2 * (1 - lay), g0[0]);
     }
   }
-  // health flags by integer tests on the bits (off the FP64 pipe)
-  int fl = 0;
-  for (int v = 0; v < NV; v++)
-    if (!finite_bits(nw[v]) || !isfinite(GGn[v][0]) || !isfinite(GGn[v][1])) fl |= 2;
-  if (!(dbits(nw[0]) > 0) || !(dbits(nw[3]) > 0)) fl |= 1;
   *flags = act ? fl : 0;
-  if (stage != 2 || !act) return 0;
-  return cfl_ratio<R>(nw, d.dX[j], G);
+  if (stage != 2) return 0;
+  R upper = speed[NL - 1], lower = speed[0];
+  if (NL == 1) {
+    const R other = __shfl_xor_sync(0xffffffffu, speed[0], 1);
+    upper = lay == 1 ? speed[0] : other;
+    lower = lay == 1 ? other : speed[0];
+  }
+  if (!act) return 0;
+  return cfl_ratio<R>(upper, lower, d.dX[j]);
 }
+#endif
 
 }  // namespace gks2l
