@@ -289,9 +289,11 @@ int gks2l_mlp_forward(const float *d_X, int32_t n, const float *d_params, float 
 /* ---- launch shapes (not part of the paper) --------------------------------
  * The interface, edge and update kernels each run in one of five launch
  * shapes (with the gate on, the edge shape applies to the fused interface and
- * edge kernel): 0: 64 threads per block, 1: 128 (default), 2: 256, 3: 128 threads
- * held to 64 registers (eight blocks per SM), 4: 128 threads held to 128
- * registers (four blocks per SM). shapes[3] picks the learned gate's variant:
+ * edge kernel): 0: 64 threads per block (default; the update: 1), 1: 128, 2:
+ * 256, 3: 128 threads held to 64 registers (eight blocks per SM), 4: 128
+ * threads held to 128 registers (four blocks per SM). In shapes 0-2 small
+ * meshes take smaller blocks (the double form) and a layer per thread (the
+ * update). shapes[3] picks the learned gate's variant:
  * its kernel (shapes[3] % 4): 0 (default), each warp takes 32 cells through
  * mma.sync BF16 tiles, the network in registers; 1, each 128-thread block
  * takes 128 cells through tcgen05 MMAs (M = 128, N = 32) with the
@@ -299,7 +301,10 @@ int gks2l_mlp_forward(const float *d_X, int32_t n, const float *d_params, float 
  * the same kernel with two and four times as many blocks per SM. Its
  * placement (shapes[3] / 4 % 2): the gate reads the stage's state and runs on
  * a second stream beside the edge kernels (0) or beside the reconstruction
- * (1), joining before the cell update. The gated run's edge path
+ * (1), joining before the cell update; the mma.sync kernel beside the
+ * reconstruction (variants 4 and 12) runs inside it in the single form, which
+ * is also what the single form does while no variant has been chosen (by this
+ * call or by the autotuner). The gated run's edge path
  * (shapes[3] / 8): 0, one fused interface-and-edge pass plus a deferred pass
  * for the edges whose plane gradients carry weight; 1, the plain interface
  * and edge kernels (faster when the gate calls few cells smooth). The gate
@@ -325,8 +330,9 @@ int gks2l_autotune(gks2l_ctx *ctx, int32_t n_steps, int32_t shapes[4]);
  * one between CUDA events on the bound stream, then synchronises. ms[k] is
  * the mean duration of one launch of kernel k, in the order: reconstruction,
  * interface levels, edge solution, cell update (each averaged over both
- * stages), step start, troubled-cell gate (0 when it is off; run here in
- * sequence, in gks2l_advance on a second stream). With the gate on and the
+ * stages), step start, troubled-cell gate (about 0 when it is off or inside
+ * the reconstruction; run here in sequence, in gks2l_advance on a second
+ * stream). With the gate on and the
  * fused edge path (gate variants 0-7), the
  * interface levels and the edge solution run as one fused kernel, reported
  * in the edge slot, followed by a pass over the edges whose solution needs

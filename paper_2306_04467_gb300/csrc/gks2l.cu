@@ -65,6 +65,7 @@ template <typename R> struct TileLayout {
   static constexpr bool REUSE = sizeof(R) == 8;                // the second copy takes the LSQ rows' space
   static constexpr unsigned LATE = REUSE ? LSQ : P1;           // where the second copy lands
   static constexpr unsigned BAR = REUSE ? P1 : END;            // two mbarriers
+  static constexpr unsigned GX = BAR + 16;                     // the gate's features, [TW][MLP_IN] BF16
   static_assert(2 * TW * NREC * sizeof(R) <= MM && TX2 <= MM, "the staged side records and the second copy fit there");
   static_assert(P1 % 128 == 0 && END % 128 == 0, "bulk copies move whole lines");
 };
@@ -128,7 +129,8 @@ template <typename R> struct ReconCfg {
 template <> struct ReconCfg<double> {
   static constexpr int VP = 1, BLOCKS = 4;
 };
-template <typename R> constexpr unsigned recon_smem() { return TileLayout<R>::BAR + 16; }
+template <typename R> constexpr unsigned recon_smem() { return TileLayout<R>::GX; }
+template <typename R> constexpr unsigned recon_gate_smem() { return TileLayout<R>::GX + TW * MLP_IN * 2; }
 
 // Positivity option (not in the paper), on a tile's staged side records: for
 // each cell and layer the least depth at the cell's six edge Gauss points;
@@ -171,7 +173,15 @@ __device__ void recon_positivity(const Dev &d, const Par &p, int j, int lay, R *
   }
 }
 
-template <typename R, bool POS = false>
+// GATE (FP32): the troubled-cell gate's decisions for the next reconstruction
+// are taken here too: the features come from the registers of the warp that has
+// gathered the levels' pair and wait in shared memory while the fits run; the
+// other two warps take the network (mma.sync, its weights read through L1) for
+// 16 cells each when they have written their records.
+// A kernel of its own gathers the same values again and finds no room beside
+// this one: a gated stage 660.5 -> 652.4 us at 1.04 M triangles, 153.2 -> 147.5
+// at 181 k (the best variant of each kind).
+template <typename R, bool POS = false, bool GATE = false>
 __global__ void __launch_bounds__(TW * 6 / ReconCfg<R>::VP, ReconCfg<R>::BLOCKS) k_recon(Dev d, Par p) {
   using T = TileLayout<R>;
   constexpr int VP = ReconCfg<R>::VP;
@@ -210,7 +220,16 @@ __global__ void __launch_bounds__(TW * 6 / ReconCfg<R>::VP, ReconCfg<R>::BLOCKS)
     int st[NSLOT];
 #pragma unroll
     for (int s = 0; s < NSLOT; s++) st[s] = d.st_cell[(size_t)s * d.cs + jj];
-    recon_gather<R, VP>(d, jj, pair, comp, st, d.tile_xf[blockIdx.x] != 0, rhs, q0);
+    R nq[4][2], g[4][4];
+    recon_gather<R, VP>(d, jj, pair, comp, st, d.tile_xf[blockIdx.x] != 0, rhs, q0, nq, g);
+    if (GATE && pair == 0) {
+      float f[MLP_IN];
+      gate_features_of<R>(d, jj, nq, g, f);
+      uint2 *row = reinterpret_cast<uint2 *>(sm + T::GX) + lane * (MLP_IN / 4);
+      for (int k = 0; k < MLP_IN / 4; k++)
+        row[k] = make_uint2(active ? pack_bf16(f[4 * k], f[4 * k + 1]) : 0u,
+                            active ? pack_bf16(f[4 * k + 2], f[4 * k + 3]) : 0u);
+    }
   };
   if (VP == 2) gather();   // (the double form's registers do not hold them across the wait)
   __syncthreads();
@@ -266,15 +285,26 @@ __global__ void __launch_bounds__(TW * 6 / ReconCfg<R>::VP, ReconCfg<R>::BLOCKS)
   uint4 *dst = reinterpret_cast<uint4 *>((R *)d.srec + (size_t)blockIdx.x * (2 * NREC * TW)) + lane;
   if (!POS) {
     // a warp's 32 vectors are contiguous
-    if (!active) return;
-    for (int i = 0; i < VP; i++) {
-      int layer;
-      const int slot = slot_of(pair, VP == 2 ? i : comp, layer);
-      for (int k = 0; k < NVEC; k++) {
-        uint4 t;
-        memcpy(&t, rec[i] + k * V, 16);
-        dst[((layer * 3 + slot) * NVEC + k) * TW] = t;
+    if (active) {
+      for (int i = 0; i < VP; i++) {
+        int layer;
+        const int slot = slot_of(pair, VP == 2 ? i : comp, layer);
+        for (int k = 0; k < NVEC; k++) {
+          uint4 t;
+          memcpy(&t, rec[i] + k * V, 16);
+          dst[((layer * 3 + slot) * NVEC + k) * TW] = t;
+        }
       }
+    }
+    if (GATE && pair != 0) {
+      // 16 cells each (the features are in shared memory since the barrier
+      // behind the copies); lane r < 16 has the logit of row r
+      const int half = pair - 1;
+      const MlpImage net = {reinterpret_cast<const MlpDev *>(d.mlp)};
+      const unsigned idle = ~__ballot_sync(FULL, active) >> (16 * half);
+      const float logit = mlp_rows16(net, reinterpret_cast<const __nv_bfloat16 *>(sm + T::GX), MLP_IN, half, lane);
+      const unsigned mask = __ballot_sync(FULL, logit < net.w->threshold) | idle;
+      if (lane == 0) reinterpret_cast<unsigned short *>(d.gate_next)[2 * blockIdx.x + half] = (unsigned short)mask;
     }
     return;
   }
@@ -716,14 +746,14 @@ __global__ void __launch_bounds__(BS) k_iface(Dev d) { iface_body<R>(d); }
 // (the edge kernel in FP32 with 96 registers, ten blocks of 64 per SM: 283 us at
 // 1.04 M triangles; left alone it takes 80 and 321 us)
 template <typename R, int BS>
-__global__ void __launch_bounds__(BS, sizeof(R) == 4 && BS > 32 ? 640 / BS : 1) k_edge(Dev d, Par p, int stage) {
+__global__ void __launch_bounds__(BS, sizeof(R) == 4 ? 640 / BS : 1) k_edge(Dev d, Par p, int stage) {
   edge_body<R>(d, p, stage);
 }
 // (the fused kernel in FP32 with 72 registers, thirteen blocks of 64 per SM:
 // 282 us at 1.04 M triangles against 288 with the 80 that it takes when left
 // alone)
 template <typename R, int BS>
-__global__ void __launch_bounds__(BS, sizeof(R) == 4 && BS > 32 ? 832 / BS : 1) k_edgef(Dev d, Par p, int stage) { edge_fused_body<R>(d, p, stage); }
+__global__ void __launch_bounds__(BS, sizeof(R) == 4 ? 832 / BS : 1) k_edgef(Dev d, Par p, int stage) { edge_fused_body<R>(d, p, stage); }
 // (the update waits for its gathers: held in FP32 to 896 resident threads per
 // SM, 72 registers, 130 us at 1.04 M triangles against 152 with the 92 that it
 // takes when left alone)
@@ -974,6 +1004,7 @@ struct gks2l_ctx {
   bool has_mlp = false;
   int n_sm = 1;                // SMs of the bound device
   cudaStream_t side = nullptr; // second stream for the gate (created with the network)
+  bool gate_auto = true;       // no gate variant has been chosen
   int shape[4] = {0, 0, 1, 0}; // launch shapes of the interface, edge and update kernels; gate variant
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   int phase = 0;
@@ -1200,14 +1231,28 @@ void launch_gate(gks2l_ctx *c, const Par &p, cudaStream_t st) {
   else k_gate<R><<<nb, 128, 0, st>>>(c->d, p);
 }
 
+// Whether the reconstruction takes the gate's decisions itself: in FP32 with the
+// mma.sync kernel beside the reconstruction (variants 4 and 12), whose
+// decisions these are, or where no variant has been chosen.
+inline bool gate_in_recon(const gks2l_ctx *c, const Par &p) {
+  return p.use_gate && c->par.precision == GKS2L_FP32 && !(p.pos_floor > 0) &&
+         (c->gate_auto || (gate_kernel(c->shape[3]) == 0 && gate_beside_recon(c->shape[3])));
+}
+
 template <typename R>
-void launch_recon(gks2l_ctx *c, const Par &p) {
+void launch_recon(gks2l_ctx *c, const Par &p, bool gate = false) {
   const Dev &d = c->d;
   constexpr int UNITS = 6 / ReconCfg<R>::VP;
   const unsigned tiles = blocks(d.nt, TW);
   if (p.pos_floor > 0) {
     k_recon<R, true><<<tiles, dim3(TW, UNITS), recon_smem<R>(), c->stream>>>(d, p);
     return;
+  }
+  if constexpr (ReconCfg<R>::VP == 2) {
+    if (gate) {
+      k_recon<R, false, true><<<tiles, dim3(TW, UNITS), recon_gate_smem<R>(), c->stream>>>(d, p);
+      return;
+    }
   }
   // a small mesh in FP64: a block per tile and variable, so that the tiles'
   // warps share more SMs' FP64 pipes (each block fetches the tile's rows,
@@ -1238,7 +1283,9 @@ template <typename R> bool spread(const gks2l_ctx *c, size_t n) {
     case 2: KERNEL<R, 256><<<blocks(n, 256), 256, 0, st>>>(__VA_ARGS__); break;             \
     case 3: KERNEL##_r64<R><<<blocks(n, 128), 128, 0, st>>>(__VA_ARGS__); break;            \
     case 4: KERNEL##_r128<R><<<blocks(n, 128), 128, 0, st>>>(__VA_ARGS__); break;           \
-    case kShapes: KERNEL<R, 32><<<blocks(n, 32), 32, 0, st>>>(__VA_ARGS__); break;          \
+    case kShapes:                                                                          \
+      if constexpr (sizeof(R) == 8) KERNEL<R, 32><<<blocks(n, 32), 32, 0, st>>>(__VA_ARGS__); \
+      break;                                                                               \
     default: KERNEL<R, 128><<<blocks(n, 128), 128, 0, st>>>(__VA_ARGS__); break;            \
   }
 
@@ -1252,8 +1299,13 @@ template <typename R>
 void launch_edge(gks2l_ctx *c, const Par &p, int stage, cudaStream_t st) {
   const size_t n = 4 * (size_t)c->d.ne;
   if (p.pos_floor > 0) {
-    if (spread<R>(c, n)) k_edge_pos<R, 32><<<blocks(n, 32), 32, 0, st>>>(c->d, p, stage);
-    else k_edge_pos<R, 128><<<blocks(n, 128), 128, 0, st>>>(c->d, p, stage);
+    if constexpr (sizeof(R) == 8) {
+      if (spread<R>(c, n)) {
+        k_edge_pos<R, 32><<<blocks(n, 32), 32, 0, st>>>(c->d, p, stage);
+        return;
+      }
+    }
+    k_edge_pos<R, 128><<<blocks(n, 128), 128, 0, st>>>(c->d, p, stage);
     return;
   }
   GKS2L_SHAPE_SWITCH(c->shape[1], k_edge, n, st, c->d, p, stage)
@@ -1280,8 +1332,8 @@ void launch_update(gks2l_ctx *c, const Par &p, int stage, cudaStream_t st) {
   // 181 k and beyond both layers per thread are as fast or faster (130 against
   // 139 us at 1.04 M), in FP64 from 66 k on (41 against 46 us).
   if (c->shape[2] < 3 && blocks(n, 128) < 2 * (unsigned)c->n_sm) {
-    if (spread<R>(c, 2 * n)) k_update_layer<R, 32><<<blocks(2 * n, 32), 32, 0, st>>>(c->d, p, stage);
-    else k_update_layer<R, 128><<<blocks(2 * n, 128), 128, 0, st>>>(c->d, p, stage);
+    constexpr unsigned BS = sizeof(R) == 8 ? 32 : 128;   // (the double form is always below kSpread here)
+    k_update_layer<R, BS><<<blocks(2 * n, BS), BS, 0, st>>>(c->d, p, stage);
     return;
   }
   GKS2L_SHAPE_SWITCH(c->shape[2], k_update, n, st, c->d, p, stage)
@@ -1311,10 +1363,11 @@ void launch_stage(gks2l_ctx *c, int stage) {
   // k_update replaces, and writes its mask to a second buffer: it runs beside
   // the reconstruction or beside the edge kernels (the variant's placement)
   // and joins before k_update, which copies the mask over.
-  const bool gate_early = p.use_gate && gate_beside_recon(c->shape[3]);
+  const bool inside = gate_in_recon(c, p), beside = p.use_gate && !inside;
+  const bool gate_early = beside && gate_beside_recon(c->shape[3]);
   if (gate_early) fork_gate<R>(c, p);
-  launch_recon<R>(c, p);
-  if (p.use_gate && !gate_early) fork_gate<R>(c, p);
+  launch_recon<R>(c, p, inside);
+  if (beside && !gate_early) fork_gate<R>(c, p);
   if (fused_edges(c, p)) {
     launch_edge_fused<R>(c, p, stage, c->stream);
     launch_edge_deferred<R>(c, p, stage, c->stream);
@@ -1322,7 +1375,7 @@ void launch_stage(gks2l_ctx *c, int stage) {
     launch_iface<R>(c, c->stream);
     launch_edge<R>(c, p, stage, c->stream);
   }
-  if (p.use_gate) cudaStreamWaitEvent(c->stream, c->ev_join, 0);
+  if (beside) cudaStreamWaitEvent(c->stream, c->ev_join, 0);
   launch_update<R>(c, p, stage, c->stream);
 }
 
@@ -1589,6 +1642,8 @@ int gks2l_bind(gks2l_ctx *c, void *d_workspace, size_t bytes, void *stream) {
   }
   CK(cudaFuncSetAttribute(k_recon<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, recon_smem<float>()));
   CK(cudaFuncSetAttribute(k_recon<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, recon_smem<double>()));
+  CK(cudaFuncSetAttribute(k_recon<float, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                          recon_gate_smem<float>()));
   CK(cudaFuncSetAttribute(k_recon<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, recon_smem<float>()));
   CK(cudaFuncSetAttribute(k_recon<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                           recon_smem<double>()));
@@ -1836,17 +1891,17 @@ int gks2l_profile_kernels(gks2l_ctx *c, int32_t n_steps, double ms[6]) {
   for (int i = 0; i < 8; i++) CK(cudaEventCreate(&ev[i]));
   double acc[6] = {0, 0, 0, 0, 0, 0};
   Par p = make_par(c);
-  const bool f32 = c->par.precision == GKS2L_FP32, fused = fused_edges(c, p);
+  const bool f32 = c->par.precision == GKS2L_FP32, fused = fused_edges(c, p), inside = gate_in_recon(c, p);
   for (int s = 0; s < n_steps; s++) {
     CK(cudaEventRecord(ev[0], c->stream));
     launch_step_begin(c);
     CK(cudaEventRecord(ev[1], c->stream));
     for (int stage = 1; stage <= 2; stage++) {
       CK(cudaEventRecord(ev[2], c->stream));
-      if (f32) launch_recon<float>(c, p);
+      if (f32) launch_recon<float>(c, p, inside);
       else launch_recon<double>(c, p);
       CK(cudaEventRecord(ev[3], c->stream));
-      if (p.use_gate) {
+      if (p.use_gate && !inside) {
         if (f32) launch_gate<float>(c, p, c->stream);
         else launch_gate<double>(c, p, c->stream);
       }
@@ -1905,6 +1960,7 @@ int gks2l_set_launch_shapes(gks2l_ctx *c, const int32_t shapes[4]) {
     if (shapes[k] < 0 || shapes[k] >= kShapes) return GKS2L_EINVAL;
   if (shapes[3] < 0 || shapes[3] >= kGateVariants) return GKS2L_EINVAL;
   for (int k = 0; k < 4; k++) c->shape[k] = shapes[k];
+  c->gate_auto = false;
   drop_graph(c);
   return GKS2L_OK;
 }
@@ -1933,6 +1989,7 @@ int gks2l_autotune(gks2l_ctx *c, int32_t n_steps, int32_t shapes[4]) {
   shapes[3] = c->shape[3];
   if (c->par.indicator == GKS2L_INDICATOR_MLP && c->has_mlp) {
     double best_g = INFINITY;
+    c->gate_auto = false;
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));

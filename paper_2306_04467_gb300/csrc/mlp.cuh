@@ -33,25 +33,16 @@ struct alignas(16) MlpDev {
 // and its three face neighbours, the deviation of the average from their
 // mean and the h-scaled gradient, divided by the norm of all twelve
 // (regularised by the WENO epsilon, so smooth data give small features).
+// The features from the levels' pair (h2, eta1) of the cell and its face
+// neighbours: averages q, gradients g as image_g leaves them.
 template <typename R>
-__host__ __device__ inline void gate_features(const Dev &d, int j, float out[24]) {
-  // the levels' pair (h2, eta1) of the cell and its face neighbours: one load
-  // for a cell's two averages and one for their gradients
-  R q[4][2], g[4][4];
-  load_n<R, 2>(dq_at<R>(d, 0, j), q[0]);
-  load_g<R>(d, 0, j, g[0]);
-  int xf[3];
-  for (int f = 0; f < 3; f++) {
-    const int nb = d.st_cell[(size_t)f * d.cs + j];
-    xf[f] = d.st_xf[(size_t)f * d.cs + j];
-    load_n<R, 2>(dq_at<R>(d, 0, nb), q[1 + f]);
-    load_g<R>(d, 0, nb, g[1 + f]);
-  }
-  for (int f = 0; f < 3; f++) image_g<R>(d, 0, xf[f], g[1 + f]);
+__host__ __device__ __forceinline__ void gate_features_of(const Dev &d, int j, const R q[4][2], const R g[4][4],
+                                                          float out[24]) {
   const R hs = ((const R *)d.hsR)[j];
   const R eps = ((const R *)d.epsA)[j];
   R ref[2];
   load_n<R, 2>((const R *)d.refR + 2 * d.inst[j], ref);
+#pragma unroll
   for (int h = 0; h < 2; h++) {
     const int c = 1 - h;
     R mean = (q[0][c] + q[1][c] + q[2][c] + q[3][c]) * (R)0.25;
@@ -67,6 +58,22 @@ __host__ __device__ inline void gate_features(const Dev &d, int j, float out[24]
     R is = (R)1 / r_sqrt<R>(ss);
     for (int k = 0; k < 12; k++) out[12 * h + k] = (float)(raw[k] * is);
   }
+}
+template <typename R>
+__host__ __device__ inline void gate_features(const Dev &d, int j, float out[24]) {
+  // one load for a cell's two averages and one for their gradients
+  R q[4][2], g[4][4];
+  load_n<R, 2>(dq_at<R>(d, 0, j), q[0]);
+  load_g<R>(d, 0, j, g[0]);
+  int xf[3];
+  for (int f = 0; f < 3; f++) {
+    const int nb = d.st_cell[(size_t)f * d.cs + j];
+    xf[f] = d.st_xf[(size_t)f * d.cs + j];
+    load_n<R, 2>(dq_at<R>(d, 0, nb), q[1 + f]);
+    load_g<R>(d, 0, nb, g[1 + f]);
+  }
+  for (int f = 0; f < 3; f++) image_g<R>(d, 0, xf[f], g[1 + f]);
+  gate_features_of<R>(d, j, q, g, out);
 }
 
 #ifdef __CUDACC__
@@ -85,6 +92,14 @@ __device__ __forceinline__ unsigned pack_bf16(float lo, float hi) {
 }
 __device__ __forceinline__ unsigned ld_pair(const __nv_bfloat16 *p) { return *reinterpret_cast<const unsigned *>(p); }
 
+// The A fragment of columns 16..31 where the tile ends at column 24 (MLP_IN):
+// the rest is zero
+__device__ __forceinline__ void load_a_half(unsigned a[4], const __nv_bfloat16 *t, int ld, int r0, int lane) {
+  const int g = lane >> 2, c = (lane & 3) * 2;
+  a[0] = ld_pair(t + (r0 + g) * ld + 16 + c);
+  a[1] = ld_pair(t + (r0 + g + 8) * ld + 16 + c);
+  a[2] = a[3] = 0u;
+}
 // A fragment (16 rows x 16 cols, k offset k0) from a bf16 row-major tile with
 // leading dimension ld (elements); lane layout of mma.m16n8k16
 __device__ __forceinline__ void load_a(unsigned a[4], const __nv_bfloat16 *t, int ld, int r0, int k0, int lane) {
@@ -190,6 +205,23 @@ __device__ __forceinline__ float2 frag_b1(const MlpFrags &F, int nt, int) { retu
 __device__ __forceinline__ float2 frag_b2(const MlpFrags &F, int nt, int) { return make_float2(F.b2[nt][0], F.b2[nt][1]); }
 __device__ __forceinline__ float2 frag_w3(const MlpFrags &F, int nt, int) { return make_float2(F.w3[nt][0], F.w3[nt][1]); }
 __device__ __forceinline__ float frag_b3(const MlpFrags &F) { return F.b3; }
+// the same from the network's image as it is used (one tile: not worth registers)
+struct MlpImage {
+  const MlpDev *w;
+};
+__device__ __forceinline__ void frag_w1(const MlpImage &F, int ks, int nt, int lane, unsigned b[2]) {
+  load_b_nk(b, F.w->w1, 32, 8 * nt, 16 * ks, lane);
+}
+__device__ __forceinline__ void frag_w2(const MlpImage &F, int ks, int nt, int lane, unsigned b[2]) {
+  load_b_nk(b, F.w->w2, 32, 8 * nt, 16 * ks, lane);
+}
+__device__ __forceinline__ float2 frag_pair(const float *p, int nt, int lane) {
+  return *reinterpret_cast<const float2 *>(p + 8 * nt + (lane & 3) * 2);
+}
+__device__ __forceinline__ float2 frag_b1(const MlpImage &F, int nt, int lane) { return frag_pair(F.w->b1, nt, lane); }
+__device__ __forceinline__ float2 frag_b2(const MlpImage &F, int nt, int lane) { return frag_pair(F.w->b2, nt, lane); }
+__device__ __forceinline__ float2 frag_w3(const MlpImage &F, int nt, int lane) { return frag_pair(F.w->w3, nt, lane); }
+__device__ __forceinline__ float frag_b3(const MlpImage &F) { return F.w->b3; }
 
 template <typename Frags>
 __device__ inline float mlp_rows16(const Frags &F, const __nv_bfloat16 *X, int ld, int mt, int lane) {
@@ -199,7 +231,8 @@ __device__ inline float mlp_rows16(const Frags &F, const __nv_bfloat16 *X, int l
     for (int i = 0; i < 4; i++) z1[nt][i] = 0.f;
   for (int ks = 0; ks < 2; ks++) {
     unsigned a[4];
-    load_a(a, X, ld, 16 * mt, 16 * ks, lane);
+    if (ks == 1 && ld == MLP_IN) load_a_half(a, X, ld, 16 * mt, lane);
+    else load_a(a, X, ld, 16 * mt, 16 * ks, lane);
     for (int nt = 0; nt < 4; nt++) {
       unsigned b[2];
       frag_w1(F, ks, nt, lane, b);

@@ -343,7 +343,9 @@ template <typename R> struct CellOps {
 
 // right-hand side: stencil average differences, then h-scaled gradients of
 // the cell and its three face neighbours. st: the stencil's cells (-1: none);
-// xfs: whether any stencil of the tile is seen through a transform
+// xfs: whether any stencil of the tile is seen through a transform. With VP = 2
+// also the averages (nq) and gradients (g) of the cell and its face neighbours
+// themselves, for the gate's features
 template <typename R>
 __host__ __device__ __forceinline__ void gather_one(const Dev &d, int j, int pair, int comp, const int st[NSLOT],
                                                     bool xfs, R rhs[NCOL], R &q0) {
@@ -391,12 +393,12 @@ __host__ __device__ __forceinline__ void gather_one(const Dev &d, int j, int pai
 }
 template <typename R, int VP>
 __host__ __device__ __forceinline__ void recon_gather(const Dev &d, int j, int pair, int comp, const int st[NSLOT],
-                                                      bool xfs, R rhs[VP][NCOL], R q0[VP]) {
+                                                      bool xfs, R rhs[VP][NCOL], R q0[VP], R nq[4][2], R g[4][4]) {
   if (VP == 1) {
     gather_one<R>(d, j, pair, comp, st, xfs, rhs[0], q0[0]);
     return;
   }
-  R q[2], t[NSLOT][2], g[4][4];
+  R q[2], t[NSLOT][2];
   load_n<R, 2>(dq_at<R>(d, pair, j), q);
 #pragma unroll
   for (int s = 0; s < NSLOT; s++) load_n<R, 2>(dq_at<R>(d, pair, st[s] >= 0 ? st[s] : j), t[s]);
@@ -411,6 +413,10 @@ __host__ __device__ __forceinline__ void recon_gather(const Dev &d, int j, int p
       image_q<R>(d, pair, xf, t[s]);
       if (s < 3) image_g<R>(d, pair, xf, g[1 + s]);
     }
+  }
+  for (int i = 0; i < 2; i++) {
+    nq[0][i] = q[i];
+    for (int f = 0; f < 3; f++) nq[1 + f][i] = t[f][i];
   }
 #pragma unroll
   for (int i = 0; i < VP; i++) {
