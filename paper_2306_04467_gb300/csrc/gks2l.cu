@@ -26,6 +26,7 @@
 
 #include "edge64.cuh"
 #include "gks2l.h"
+#include "launch.cuh"
 #include "mlp.cuh"
 #include "prep.h"
 #include "stage.cuh"
@@ -192,6 +193,7 @@ __global__ void __launch_bounds__(TW * 6 / ReconCfg<R>::VP, ReconCfg<R>::BLOCKS)
   // tile's cells it calls smooth; a tile whose cells all take the linear
   // weights needs neither the P1 rows nor the smoothness forms
   const bool gate_on = p.use_gate && !p.harvest;
+  dep_wait();
   const unsigned lin_mask = gate_on ? d.gate_mask[blockIdx.x] : 0u;
   const bool all_linear = lin_mask == 0xffffffffu;
   if (lane == 0 && threadIdx.y == 0) {
@@ -576,6 +578,7 @@ __device__ __forceinline__ void edge_write(const Dev &d, int e, int ell, int q, 
 
 template <typename R>
 __device__ __forceinline__ void iface_body(const Dev &d) {
+  dep_wait();
   int tid = blockIdx.x * blockDim.x + threadIdx.x;
   if constexpr (sizeof(R) == 8) {
     // every thread computes (past the last edge: the last edge again): lanes
@@ -592,6 +595,7 @@ __device__ __forceinline__ void iface_body(const Dev &d) {
 
 template <typename R, bool POS = false>
 __device__ __forceinline__ void edge_body(const Dev &d, const Par &p, int stage) {
+  dep_wait();
   int tid = blockIdx.x * blockDim.x + threadIdx.x;
   int e = tid >> 2, ell = (tid >> 1) & 1, q = tid & 1;
   const int ee = e < d.ne ? e : d.ne - 1;
@@ -615,6 +619,7 @@ __device__ __forceinline__ void edge_body(const Dev &d, const Par &p, int stage)
 // worklist for k_edge_deferred, which runs once every blended level exists.
 template <typename R>
 __device__ __forceinline__ void edge_fused_body(const Dev &d, const Par &p, int stage) {
+  dep_wait();
   int tid = blockIdx.x * blockDim.x + threadIdx.x;
   int e = tid >> 2, ell = (tid >> 1) & 1, q = tid & 1;
   const int ee = e < d.ne ? e : d.ne - 1;
@@ -654,6 +659,7 @@ constexpr int DEFER_BLOCKS_PER_SM = 4;
 
 template <typename R>
 __global__ void __launch_bounds__(128) k_edge_deferred(Dev d, Par p, int stage) {
+  dep_wait();
   const int n = *d.wl_count;
   const int lane = threadIdx.x & 31;
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarp = (gridDim.x * blockDim.x) >> 5;
@@ -723,6 +729,7 @@ __global__ void k_mass(Dev d) {
 
 template <typename R, int NL = 2>
 __device__ __forceinline__ void update_body(const Dev &d, const Par &p, int stage) {
+  dep_wait();
   const int tid = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = NL == 2 ? tid : tid >> 1, lay = NL == 2 ? 0 : tid & 1, jj = j < d.nt ? j : d.nt - 1;
   const bool ok = j < d.nt;
@@ -798,6 +805,7 @@ template <typename R>
 __global__ void __launch_bounds__(REF_THREADS) k_ref(Dev d, const int *chunk, const int *inst_chunk, double *part) {
   __shared__ double sh[3][REF_THREADS];
   __shared__ bool last;
+  dep_wait();
   const int c = blockIdx.x, t = threadIdx.x, j1 = chunk[2 * c + 1];
   double a = 0, s2 = 0, s1 = 0;
   for (int j = chunk[2 * c] + t; j < j1; j += REF_THREADS) {
@@ -875,6 +883,7 @@ __global__ void k_step_begin(Dev d, Par p, const double *tend) {
 // a clear mask. Edges: R1 - B at the Gauss points.
 template <typename R>
 __global__ void __launch_bounds__(128) k_init(Dev d, Par p, const int *perm, const double *grad_caller) {
+  dep_wait();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j < d.ne) {
     const double R1 = d.ref[2 * d.eg[4 * (size_t)j + 3] + 1];
@@ -1240,17 +1249,17 @@ inline bool gate_in_recon(const gks2l_ctx *c, const Par &p) {
 }
 
 template <typename R>
-void launch_recon(gks2l_ctx *c, const Par &p, bool gate = false) {
+void launch_recon(gks2l_ctx *c, const Par &p, bool gate = false, bool chained = false) {
   const Dev &d = c->d;
   constexpr int UNITS = 6 / ReconCfg<R>::VP;
   const unsigned tiles = blocks(d.nt, TW);
   if (p.pos_floor > 0) {
-    k_recon<R, true><<<tiles, dim3(TW, UNITS), recon_smem<R>(), c->stream>>>(d, p);
+    launch(chained, k_recon<R, true>, tiles, dim3(TW, UNITS), recon_smem<R>(), c->stream, d, p);
     return;
   }
   if constexpr (ReconCfg<R>::VP == 2) {
     if (gate) {
-      k_recon<R, false, true><<<tiles, dim3(TW, UNITS), recon_gate_smem<R>(), c->stream>>>(d, p);
+      launch(chained, k_recon<R, false, true>, tiles, dim3(TW, UNITS), recon_gate_smem<R>(), c->stream, d, p);
       return;
     }
   }
@@ -1258,7 +1267,8 @@ void launch_recon(gks2l_ctx *c, const Par &p, bool gate = false) {
   // warps share more SMs' FP64 pipes (each block fetches the tile's rows,
   // from L2); from one tile per SM on all pipes have work anyway
   const bool split = sizeof(R) == 8 && tiles < (unsigned)c->n_sm;
-  k_recon<R><<<dim3(tiles, split ? UNITS : 1), dim3(TW, split ? 1 : UNITS), recon_smem<R>(), c->stream>>>(d, p);
+  launch(chained, k_recon<R>, dim3(tiles, split ? UNITS : 1), dim3(TW, split ? 1 : UNITS), recon_smem<R>(), c->stream, d,
+         p);
 }
 
 // launch shapes the autotuner chooses from: 0: 64 threads, 1: 128 threads,
@@ -1277,22 +1287,22 @@ template <typename R> bool spread(const gks2l_ctx *c, size_t n) {
   return sizeof(R) == 8 && blocks(n, 128) < kSpread * (unsigned)c->n_sm;
 }
 
-#define GKS2L_SHAPE_SWITCH(cfg, KERNEL, n, st, ...)                                          \
-  switch (cfg < 3 && spread<R>(c, n) ? kShapes : cfg) {                                    \
-    case 0: KERNEL<R, 64><<<blocks(n, 64), 64, 0, st>>>(__VA_ARGS__); break;                \
-    case 2: KERNEL<R, 256><<<blocks(n, 256), 256, 0, st>>>(__VA_ARGS__); break;             \
-    case 3: KERNEL##_r64<R><<<blocks(n, 128), 128, 0, st>>>(__VA_ARGS__); break;            \
-    case 4: KERNEL##_r128<R><<<blocks(n, 128), 128, 0, st>>>(__VA_ARGS__); break;           \
-    case kShapes:                                                                          \
-      if constexpr (sizeof(R) == 8) KERNEL<R, 32><<<blocks(n, 32), 32, 0, st>>>(__VA_ARGS__); \
-      break;                                                                               \
-    default: KERNEL<R, 128><<<blocks(n, 128), 128, 0, st>>>(__VA_ARGS__); break;            \
+#define GKS2L_SHAPE_SWITCH(chained, cfg, KERNEL, n, st, ...)                                            \
+  switch (cfg < 3 && spread<R>(c, n) ? kShapes : cfg) {                                                \
+    case 0: launch(chained, KERNEL<R, 64>, blocks(n, 64), 64, 0, st, __VA_ARGS__); break;               \
+    case 2: launch(chained, KERNEL<R, 256>, blocks(n, 256), 256, 0, st, __VA_ARGS__); break;            \
+    case 3: launch(chained, KERNEL##_r64<R>, blocks(n, 128), 128, 0, st, __VA_ARGS__); break;           \
+    case 4: launch(chained, KERNEL##_r128<R>, blocks(n, 128), 128, 0, st, __VA_ARGS__); break;          \
+    case kShapes:                                                                                      \
+      if constexpr (sizeof(R) == 8) launch(chained, KERNEL<R, 32>, blocks(n, 32), 32, 0, st, __VA_ARGS__); \
+      break;                                                                                           \
+    default: launch(chained, KERNEL<R, 128>, blocks(n, 128), 128, 0, st, __VA_ARGS__); break;           \
   }
 
 template <typename R>
 void launch_iface(gks2l_ctx *c, cudaStream_t st) {
   const size_t n = (sizeof(R) == 8 ? 4 : 2) * (size_t)c->d.ne;
-  GKS2L_SHAPE_SWITCH(c->shape[0], k_iface, n, st, c->d)
+  GKS2L_SHAPE_SWITCH(true, c->shape[0], k_iface, n, st, c->d)
 }
 
 template <typename R>
@@ -1301,14 +1311,14 @@ void launch_edge(gks2l_ctx *c, const Par &p, int stage, cudaStream_t st) {
   if (p.pos_floor > 0) {
     if constexpr (sizeof(R) == 8) {
       if (spread<R>(c, n)) {
-        k_edge_pos<R, 32><<<blocks(n, 32), 32, 0, st>>>(c->d, p, stage);
+        launch(true, k_edge_pos<R, 32>, blocks(n, 32), 32, 0, st, c->d, p, stage);
         return;
       }
     }
-    k_edge_pos<R, 128><<<blocks(n, 128), 128, 0, st>>>(c->d, p, stage);
+    launch(true, k_edge_pos<R, 128>, blocks(n, 128), 128, 0, st, c->d, p, stage);
     return;
   }
-  GKS2L_SHAPE_SWITCH(c->shape[1], k_edge, n, st, c->d, p, stage)
+  GKS2L_SHAPE_SWITCH(true, c->shape[1], k_edge, n, st, c->d, p, stage)
 }
 
 // gated runs: interface levels and edge solution fused, then the deferred
@@ -1316,15 +1326,15 @@ void launch_edge(gks2l_ctx *c, const Par &p, int stage, cudaStream_t st) {
 template <typename R>
 void launch_edge_fused(gks2l_ctx *c, const Par &p, int stage, cudaStream_t st) {
   const size_t n = 4 * (size_t)c->d.ne;
-  GKS2L_SHAPE_SWITCH(c->shape[1], k_edgef, n, st, c->d, p, stage)
+  GKS2L_SHAPE_SWITCH(true, c->shape[1], k_edgef, n, st, c->d, p, stage)
 }
 template <typename R>
 void launch_edge_deferred(gks2l_ctx *c, const Par &p, int stage, cudaStream_t st) {
-  k_edge_deferred<R><<<c->n_sm * DEFER_BLOCKS_PER_SM, 128, 0, st>>>(c->d, p, stage);
+  launch(true, k_edge_deferred<R>, c->n_sm * DEFER_BLOCKS_PER_SM, 128, 0, st, c->d, p, stage);
 }
 
 template <typename R>
-void launch_update(gks2l_ctx *c, const Par &p, int stage, cudaStream_t st) {
+void launch_update(gks2l_ctx *c, const Par &p, int stage, cudaStream_t st, bool chained = false) {
   const size_t n = (size_t)c->d.nt;
   // A mesh that does not fill the SMs' threads is bound by the length of one
   // thread's chain of loads (and in FP64 of its FP64 operations): a layer per
@@ -1333,10 +1343,10 @@ void launch_update(gks2l_ctx *c, const Par &p, int stage, cudaStream_t st) {
   // 139 us at 1.04 M), in FP64 from 66 k on (41 against 46 us).
   if (c->shape[2] < 3 && blocks(n, 128) < 2 * (unsigned)c->n_sm) {
     constexpr unsigned BS = sizeof(R) == 8 ? 32 : 128;   // (the double form is always below kSpread here)
-    k_update_layer<R, BS><<<blocks(2 * n, BS), BS, 0, st>>>(c->d, p, stage);
+    launch(chained, k_update_layer<R, BS>, blocks(2 * n, BS), BS, 0, st, c->d, p, stage);
     return;
   }
-  GKS2L_SHAPE_SWITCH(c->shape[2], k_update, n, st, c->d, p, stage)
+  GKS2L_SHAPE_SWITCH(chained, c->shape[2], k_update, n, st, c->d, p, stage)
 }
 
 // With the gate on, the interface levels and the edge solution run as one
@@ -1357,7 +1367,7 @@ void fork_gate(gks2l_ctx *c, const Par &p) {
 }
 
 template <typename R>
-void launch_stage(gks2l_ctx *c, int stage) {
+void launch_stage(gks2l_ctx *c, int stage, bool chained) {
   Par p = make_par(c);
   // The gate for the next stage reads this stage's state, which only
   // k_update replaces, and writes its mask to a second buffer: it runs beside
@@ -1366,7 +1376,7 @@ void launch_stage(gks2l_ctx *c, int stage) {
   const bool inside = gate_in_recon(c, p), beside = p.use_gate && !inside;
   const bool gate_early = beside && gate_beside_recon(c->shape[3]);
   if (gate_early) fork_gate<R>(c, p);
-  launch_recon<R>(c, p, inside);
+  launch_recon<R>(c, p, inside, chained);
   if (beside && !gate_early) fork_gate<R>(c, p);
   if (fused_edges(c, p)) {
     launch_edge_fused<R>(c, p, stage, c->stream);
@@ -1376,12 +1386,13 @@ void launch_stage(gks2l_ctx *c, int stage) {
     launch_edge<R>(c, p, stage, c->stream);
   }
   if (beside) cudaStreamWaitEvent(c->stream, c->ev_join, 0);
-  launch_update<R>(c, p, stage, c->stream);
+  launch_update<R>(c, p, stage, c->stream, !beside);
 }
 
-void launch_stage_any(gks2l_ctx *c, int stage) {
-  if (c->par.precision == GKS2L_FP32) launch_stage<float>(c, stage);
-  else launch_stage<double>(c, stage);
+// (chained: a kernel of the same call precedes the stage)
+void launch_stage_any(gks2l_ctx *c, int stage, bool chained = false) {
+  if (c->par.precision == GKS2L_FP32) launch_stage<float>(c, stage, chained);
+  else launch_stage<double>(c, stage, chained);
 }
 
 void launch_step_begin(gks2l_ctx *c) {
@@ -1410,8 +1421,8 @@ int ensure_graph(gks2l_ctx *c) {
   CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
   c->stream = st;
   launch_step_begin(c);
-  launch_stage_any(c, 1);
-  launch_stage_any(c, 2);
+  launch_stage_any(c, 1, true);
+  launch_stage_any(c, 2, true);
   c->stream = user;
   cudaError_t e = cudaStreamEndCapture(st, &c->graph);
   if (e != cudaSuccess) {
@@ -1452,8 +1463,8 @@ int check_status(gks2l_ctx *c) {
 
 template <typename R>
 void launch_init(gks2l_ctx *c, const Par &p, const double *grad_caller) {
-  k_ref<R><<<c->nchunk, REF_THREADS, 0, c->stream>>>(c->d, c->d_chunk, c->d_inst_chunk, c->d_refpart);
-  k_init<R><<<blocks(std::max(c->d.nt, c->d.ne), 128), 128, 0, c->stream>>>(c->d, p, c->d_perm, grad_caller);
+  launch(true, k_ref<R>, c->nchunk, REF_THREADS, 0, c->stream, c->d, c->d_chunk, c->d_inst_chunk, c->d_refpart);
+  launch(true, k_init<R>, blocks(std::max(c->d.nt, c->d.ne), 128), 128, 0, c->stream, c->d, p, c->d_perm, grad_caller);
   if (p.use_gate) {
     // the gate's decisions on the state just set serve the first
     // reconstruction (every cell counts as active: no dt is known yet)

@@ -17,6 +17,7 @@
 #include <mutex>
 
 #include "gks2l.h"
+#include "launch.cuh"
 #include "mlp.cuh"
 
 using namespace gks2l;
@@ -301,6 +302,7 @@ __global__ void __launch_bounds__(TPB) k_mlp_grad(const float *X, const float *y
 constexpr int RED_COLS = 32, RED_ROWS = 8;
 __global__ void __launch_bounds__(RED_COLS *RED_ROWS) k_mlp_reduce(const float *part, int nparts, float *grads,
                                                                    float *loss_out) {
+  dep_wait();
   __shared__ float s[RED_ROWS][RED_COLS];
   const int col = threadIdx.x % RED_COLS, row = threadIdx.x / RED_COLS, i = blockIdx.x * RED_COLS + col;
   float v = 0.f;
@@ -381,29 +383,15 @@ constexpr int MAX_DEV = 64;
 struct PerDevice {
   std::once_flag once;
   int sms = 0;
-  cudaMemPool_t pool = nullptr;
 };
 PerDevice g_dev[MAX_DEV];
 
-// The partial sums' memory comes stream-ordered from a pool of the library's
-// own that keeps up to kPoolKeep bytes (the largest call's) between calls: the
-// device's default pool gives everything back at each synchronisation, and
-// mapping it again took 170 us of a call that follows one. Safe for any
-// number of threads and streams, as cudaMallocAsync is.
-constexpr uint64_t kPoolKeep = 4u << 20;
 PerDevice *this_device() {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAX_DEV) return nullptr;
   PerDevice &D = g_dev[dev];
   std::call_once(D.once, [&] {
     if (cudaDeviceGetAttribute(&D.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) D.sms = 0;
-    cudaMemPoolProps props = {};
-    props.allocType = cudaMemAllocationTypePinned;
-    props.location.type = cudaMemLocationTypeDevice;
-    props.location.id = dev;
-    uint64_t keep = kPoolKeep;
-    if (cudaMemPoolCreate(&D.pool, &props) != cudaSuccess) D.pool = nullptr;
-    else cudaMemPoolSetAttribute(D.pool, cudaMemPoolAttrReleaseThreshold, &keep);
   });
   return D.sms > 0 ? &D : nullptr;
 }
@@ -421,11 +409,10 @@ extern "C" int gks2l_mlp_grad(const float *d_X, const float *d_y, int32_t n, con
   const unsigned grid = grid_for(n, 16 * (TPB / 32), 2 * D->sms);
   const size_t bytes = (size_t)grid * NPART * sizeof(float);
   float *part = nullptr;
-  if ((D->pool ? cudaMallocFromPoolAsync((void **)&part, bytes, D->pool, s) : cudaMallocAsync((void **)&part, bytes, s)) !=
-      cudaSuccess)
-    return GKS2L_ECUDA;
+  if (cudaMallocAsync((void **)&part, bytes, s) != cudaSuccess) return GKS2L_ECUDA;
   k_mlp_grad<<<grid, TPB, 0, s>>>(d_X, d_y, n, d_params, pos_weight, part);
-  k_mlp_reduce<<<(NPART + RED_COLS - 1) / RED_COLS, RED_COLS * RED_ROWS, 0, s>>>(part, (int)grid, d_grads, d_loss);
+  launch(true, k_mlp_reduce, (NPART + RED_COLS - 1) / RED_COLS, RED_COLS * RED_ROWS, 0, s, part, (int)grid, d_grads,
+         d_loss);
   const bool ok = cudaGetLastError() == cudaSuccess;
   if (cudaFreeAsync(part, s) != cudaSuccess || !ok) return GKS2L_ECUDA;
   return GKS2L_OK;
