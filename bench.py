@@ -119,12 +119,13 @@ WORK_PER_UNIT = {
 # FP32 flops per unit that the hardware executes (ncu sm__sass_thread_inst_
 # executed_op_f{add,mul,fma} with FMA = 2): reported beside the algorithmic
 # counts as the overhead ratio. recon, gate, edge_fused, update: one step of
-# the large configuration at 1416 x 177 squares (501,264 triangles), the
-# current kernels; iface and edge (the plain form's): the lake at 512 x 512
-# squares, captured before the edge kernels' last instruction cuts.
+# the large configuration at 1416 x 177 squares (501,264 triangles); iface and
+# edge (the plain form's): the lake at 512 x 512 squares, captured before the
+# edge kernels' last instruction cuts. The FP32 arithmetic has not changed
+# since these captures; its loads, stores and launches have.
 EXECUTED_FP32_PER_UNIT = {"recon": 2214, "gate": 258, "iface": 836, "edge": 5405, "edge_fused": 5500,
                           "update": 319}
-# Measured FMA-chain peaks of this GB300 pool (TFLOP/s, 2 flops per FMA); the
+# Measured FMA-chain peaks of a GB300 (TFLOP/s, 2 flops per FMA); the
 # bench replaces them with the same run's own measurement.
 PEAK_TFLOPS = {"fp32": 76.5, "fp64": 1.254}
 # DRAM bytes per unit (dram__bytes_read.sum + dram__bytes_write.sum of the
@@ -132,7 +133,7 @@ PEAK_TFLOPS = {"fp32": 76.5, "fp64": 1.254}
 # current kernels on the large configuration at 1416 x 177 squares (inputs
 # larger than L2); the bench scales them to its launch by the units. A kernel
 # is listed only while it is unchanged since that capture.
-TRAFFIC_PER_UNIT = {"recon": 1040.0, "gate": 59.1, "edge_fused": 362.5, "update": 461.3}
+TRAFFIC_PER_UNIT = {"recon": 1017.0, "edge_fused": 362.7, "update": 486.0}
 
 
 KERNEL_NAME = {"edge_fused": "k_edgef", "edge_deferred": "k_edge_deferred"}
@@ -647,7 +648,9 @@ def main():
     timed = [x for x in kern if x != "step_begin"]
     ksum = sum(kern[x] for x in timed)
     share = {x: kern[x] / ksum for x in timed}
-    launches_per_step = 1 + 2 * 5   # step start + (reconstruction, gate, fused edge, deferred edges, update) per stage
+    # step start, then per stage reconstruction, two edge kernels, update and,
+    # unless the reconstruction takes its decisions (variants 4 and 12), the gate
+    launches_per_step = 1 + 2 * (4 if rh["shapes"][3] in (4, 12) else 5)
 
     def strip(w):
         return {"workload": w["workload"], "n_tri": w["n_tri"],

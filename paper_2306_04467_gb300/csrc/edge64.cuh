@@ -8,8 +8,8 @@
 // fewest (measured with 501 k triangles, 752 k edges): 1211 -> 777 per edge,
 // layer and point (k_edge<double> 6595 -> 4274 us) and 341 -> 274 per edge and
 // layer (k_iface<double> 954 -> 763 us), then, with the sides' values kept by
-// k_iface and the results rotated once per edge, k_edge<double> 582 -> 496 us
-// at 65,522 triangles:
+// k_iface and the results rotated once per edge, 633 (k_edge<double> 582 -> 496
+// us at 65,522 triangles):
 //   - face-frame evaluation: the derivatives are formed along n and t at
 //     once, a mirrored side through the frame that its cell sees;
 //   - half-space moments split into a full-space and a boundary part, and the
