@@ -852,6 +852,9 @@ __global__ void __launch_bounds__(REF_THREADS) k_ref(Dev d, const int *chunk, co
   }
 }
 
+// the end time the steps read
+__global__ void k_set_tend(double *tend, double t) { *tend = t; }
+
 // step size of each instance from the CFL ratio of the current state (Sec. 4),
 // shortened to land on t_end
 template <typename R>
@@ -1006,6 +1009,7 @@ struct gks2l_ctx {
   int *d_perm = nullptr;
   double *d_tend = nullptr;
   double tend = NAN;           // the value there (NaN: unknown)
+  bool captured = false;       // a caller has captured a call, whose graph may store another value there
   cudaStream_t cap = nullptr;  // the step is captured on it when the caller's stream is the legacy one
   double *d_stage = nullptr;   // 18 * nt staging for permutations
   int nchunk = 0;              // reference-level reduction: chunks of one instance's cells
@@ -1436,14 +1440,19 @@ int ensure_graph(gks2l_ctx *c) {
   return 0;
 }
 
-// the end time the steps read (0: none), copied when it changes (a copy that a
-// capture only recorded leaves the value unknown)
+// The end time the steps read (0: none). The kernel that stores it carries it by
+// value, so that a capture of the caller's stream keeps the value of its own
+// call. Without captures the store is left out while the value stays the same;
+// a captured graph stores its value whenever it is replayed, so from a
+// context's first capture on every call stores its own.
 int set_tend(gks2l_ctx *c, double t_end) {
-  if (c->tend == t_end) return 0;
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (c->stream) CK(cudaStreamIsCapturing(c->stream, &cs));
-  CK(cudaMemcpyAsync(c->d_tend, &t_end, sizeof(double), cudaMemcpyHostToDevice, c->stream));
-  c->tend = cs == cudaStreamCaptureStatusNone ? t_end : NAN;
+  if (cs != cudaStreamCaptureStatusNone) c->captured = true;
+  if (!c->captured && c->tend == t_end) return 0;
+  k_set_tend<<<1, 1, 0, c->stream>>>(c->d_tend, t_end);
+  CK(cudaGetLastError());
+  c->tend = t_end;
   return 0;
 }
 
