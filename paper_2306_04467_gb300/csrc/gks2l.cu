@@ -856,7 +856,8 @@ __global__ void __launch_bounds__(REF_THREADS) k_ref(Dev d, const int *chunk, co
 __global__ void k_set_tend(double *tend, double t) { *tend = t; }
 
 // step size of each instance from the CFL ratio of the current state (Sec. 4),
-// shortened to land on t_end
+// shortened to land on t_end; an instance that has arrived keeps its ratio, which
+// no stage forms again while it stands, for the step to a later end time
 template <typename R>
 __global__ void k_step_begin(Dev d, Par p, const double *tend) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -864,9 +865,11 @@ __global__ void k_step_begin(Dev d, Par p, const double *tend) {
   double r = __longlong_as_double((long long)d.dtbits[i]);
   double dt = p.cfl * r;
   double te = *tend;
+  bool arrived = false;
   if (te > 0) {
     double rem = te - d.t[i];
-    if (rem <= 1e-12 * fmax(1.0, fabs(te))) dt = 0;
+    arrived = rem <= 1e-12 * fmax(1.0, fabs(te));
+    if (arrived) dt = 0;
     else if (dt > rem) dt = rem;
   }
   if (!isfinite(dt) || dt < 0) {
@@ -876,7 +879,7 @@ __global__ void k_step_begin(Dev d, Par p, const double *tend) {
   d.dt[i] = dt;
   ((R *)d.dtR)[i] = (R)dt;
   ((R *)d.dtR)[d.ninst + i] = dt > 0 ? (R)(1 / dt) : (R)0;
-  d.dtbits[i] = DBL_INF_BITS;
+  if (!arrived) d.dtbits[i] = DBL_INF_BITS;
 }
 
 // A freshly set state, one thread per cell and per edge. Cells: the deviation
