@@ -1014,7 +1014,7 @@ struct gks2l_ctx {
   double tend = NAN;           // the value there (NaN: unknown)
   bool captured = false;       // a caller has captured a call, whose graph may store another value there
   cudaStream_t cap = nullptr;  // the step is captured on it when the caller's stream is the legacy one
-  double *d_stage = nullptr;   // 18 * nt staging for permutations
+  double *d_stage = nullptr;   // scratch (layout): 18 * nt staging for permutations among others
   int nchunk = 0;              // reference-level reduction: chunks of one instance's cells
   int *d_chunk = nullptr;      // [nchunk][2] first and end cell of each chunk
   int *d_inst_chunk = nullptr; // [ninst + 1] first chunk of each instance
@@ -1051,15 +1051,12 @@ size_t layout(gks2l_ctx *c, char *base) {
   d.nt = P.nt; d.ne = P.ne; d.ninst = P.ninst; d.cs = (int)cs;
   d.inst = k.take<int>(nt);
   d.area = k.take<double>(nt);
-  d.hs = k.take<double>(nt);
   d.dX = k.take<double>(nt);
   d.hsR = k.take<char>(rs * nt);
   d.ihsR = k.take<char>(rs * nt);
   d.epsA = k.take<char>(rs * nt);
   d.bgR = k.take<char>(rs * 2 * cs);
   d.bmean = k.take<double>(nt);
-  d.bgx = k.take<double>(nt);
-  d.bgy = k.take<double>(nt);
   d.st_cell = k.take<int>(kSlots * cs);
   d.st_xf = k.take<int8_t>(kSlots * cs);
   d.tile_xf = k.take<int>(cs / TW);
@@ -1067,24 +1064,24 @@ size_t layout(gks2l_ctx *c, char *base) {
   d.plane = k.take<char>(rs * 6 * cs);
   d.cedge = k.take<int>(3 * cs);
   d.fsl = k.take<double>(3 * cs);
-  d.fslR = k.take<char>(rs * 3 * cs);
+  d.fslR = rs == 8 ? (const void *)d.fsl : k.take<char>(rs * 3 * cs);
   d.inst_first = k.take<int>(ni + 1);
   d.avg = k.take<double>(6 * cs);
   d.dq = k.take<char>(rs * 6 * cs);
   d.dg = k.take<char>(rs * 12 * cs);
   d.hrefc = k.take<char>(rs * nt);
-  d.Wn = k.take<double>(6 * cs);
-  d.Ln = k.take<double>(6 * cs);
-  d.Ltn = k.take<double>(6 * cs);
+  if (rs == 4) d.Wn = k.take<double>(6 * cs);
+  d.Ln = k.take<double>(2 * cs);
+  d.Ltn = k.take<double>(2 * cs);
   d.incR = k.take<char>(rs * 4 * cs);
   d.srec = k.take<char>(rs * 2 * NREC * cs);
   d.omg = k.take<char>(rs * 2 * cs);
   d.mlp = k.take<MlpDev>(1);
   d.gate_mask = k.take<unsigned>(cs / TW);
   d.gate_next = k.take<unsigned>(cs / TW);
-  d.pos_flag = k.take<unsigned char>(2 * cs);
-  d.pos_hbar = k.take<char>(rs * 2 * cs);
-  d.wdev = k.take<float>(6 * cs);
+  const size_t pos = c->par.positivity_floor > 0 ? 2 * cs : 0;
+  d.pos_flag = k.take<unsigned char>(pos);
+  d.pos_hbar = k.take<char>(rs * pos);
   d.eg = k.take<int>(4 * ne);
   d.en = k.take<char>(rs * 2 * ne);
   d.eb0 = k.take<double>(ne);
@@ -1092,8 +1089,6 @@ size_t layout(gks2l_ctx *c, char *base) {
   d.exi = k.take<char>(rs * 8 * ne);
   d.hrefe = k.take<char>(rs * 2 * ne);
   d.hc = k.take<char>(rs * 2 * ne);
-  d.ept = k.take<double>(rs == 8 ? 32 * ne : 0);
-  d.wl = k.take<int>(2 * ne);
   d.wl_count = k.take<int>(1);
   d.eF = k.take<char>(rs * 8 * ne);
   d.eM = k.take<double>(4 * ne);
@@ -1113,7 +1108,19 @@ size_t layout(gks2l_ctx *c, char *base) {
   d.xf = k.take<double>(4 * kMaxXf);
   c->d_perm = k.take<int>(nt);
   c->d_tend = k.take<double>(1);
-  c->d_stage = k.take<double>(18 * nt);
+  // One piece of scratch for what is never alive at the same time, all of it
+  // used on the bound stream only: the caller's state on its way in or out and
+  // the weights' departures between a harvest's two kernels (the first `own`
+  // doubles; both also between the stages of a step); the units between the fused
+  // edge pass and the deferred one; and, between the double form's interface
+  // and edge kernels, the sides' values, which take W*'s place as well: the first
+  // stage's update writes W* after them and the second stage does not read it.
+  const size_t own = std::max(18 * nt, 3 * cs);
+  c->d_stage = k.take<double>(rs == 8 ? std::max(own + 6 * cs, 32 * ne) : std::max(own, ne));
+  if (rs == 8) d.Wn = c->d_stage + own;
+  d.ept = c->d_stage;
+  d.wl = (int *)c->d_stage;
+  d.wdev = (float *)c->d_stage;
   // at most one chunk per instance plus one per REF_CHUNK cells (the sizes
   // only: the workspace size is asked for before the instances are known)
   const size_t max_chunks = ni + nt / REF_CHUNK + 1;
@@ -1197,8 +1204,7 @@ int upload_bathymetry(gks2l_ctx *c) {
     bg[2 * j + 1] = by[j];
   }
   int rc;
-  if ((rc = upload(c, c->d.bmean, bm)) || (rc = upload(c, c->d.bgx, bx)) || (rc = upload(c, c->d.bgy, by)) ||
-      (rc = upload(c, c->d.eb0, e0)) || (rc = upload(c, c->d.eb1, e1)) ||
+  if ((rc = upload(c, c->d.bmean, bm)) || (rc = upload(c, c->d.eb0, e0)) || (rc = upload(c, c->d.eb1, e1)) ||
       (rc = upload_form(c, c->d.bgR, bg, 1, false)))
     return rc;
   return 0;
@@ -1575,6 +1581,7 @@ int gks2l_workspace_bytes(const gks2l_ctx *ctx, size_t *bytes) {
   tmp.prep.ne = ctx->prep.ne;
   tmp.prep.ninst = ctx->prep.ninst;
   tmp.rsize = ctx->rsize;
+  tmp.par = ctx->par;
   *bytes = layout(&tmp, nullptr);
   return GKS2L_OK;
 }
@@ -1625,11 +1632,11 @@ int gks2l_bind(gks2l_ctx *c, void *d_workspace, size_t bytes, void *stream) {
   std::copy(P.xf.begin(), P.xf.end(), xf.begin());
   int rc;
   if ((rc = upload(c, c->d.inst, P.inst)) || (rc = upload(c, c->d.area, P.area)) ||
-      (rc = upload(c, c->d.hs, P.hs)) || (rc = upload(c, c->d.dX, P.dX)) ||
+      (rc = upload(c, c->d.dX, P.dX)) ||
       (rc = upload_rows<int>(c, c->d.st_cell, P.st_cell, kSlots)) ||
       (rc = upload_rows<int8_t>(c, c->d.st_xf, P.st_xf, kSlots)) || (rc = upload(c, c->d.tile_xf, txf)) ||
       (rc = upload_rows<int>(c, c->d.cedge, P.cedge, 3)) || (rc = upload_rows<double>(c, c->d.fsl, fsl, 3)) ||
-      (rc = upload_form(c, c->d.fslR, fsl, 3, true)) ||
+      (c->rsize == 4 && (rc = upload_form(c, c->d.fslR, fsl, 3, true))) ||
       (rc = upload(c, c->d.inst_first, P.inst_first)) || (rc = upload(c, c->d.eg, eg)) ||
       (rc = upload(c, c->d.xf, xf)) ||
       (rc = upload(c, c->d_perm, P.perm)) ||

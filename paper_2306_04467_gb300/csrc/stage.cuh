@@ -60,11 +60,11 @@ struct Dev {
   int cs;                   // stride of per-cell arrays (nt rounded up to 32)
   // per cell
   const int *inst;
-  const double *area, *hs, *dX;
+  const double *area, *dX;
   const void *hsR, *ihsR;   // sqrt|Omega| and its inverse, type R
   const void *epsA;         // weno_eps * |Omega|, type R
   const void *bgR;          // [cell][2] grad B, type R
-  const double *bmean, *bgx, *bgy;
+  const double *bmean;
   const int *st_cell;
   const int8_t *st_xf;
   const int *tile_xf;       // per tile of 32 cells: whether any of its stencils has an image transform
@@ -72,13 +72,13 @@ struct Dev {
   const void *plane;        // [(f*2+d)][cell] plane operator, type R
   const int *cedge;         // [f][cell]: edge id, or ~edge when the cell is the R side
   const double *fsl;        // [f][cell]: sign * |Gamma| / |Omega| (double, mass sums)
-  const void *fslR;         // the same, type R (the other residuals)
+  const void *fslR;         // the same, type R (the other residuals; fsl itself in the double form)
   const int *inst_first;
   double *avg;              // state averages [v][cell] (FP64)
   void *dq, *dg;            // deviation mirrors [pair][cell][2] and gradients [pair][cell][2][2], type R
   void *hrefc;              // R1 - B_j per cell, type R
-  double *Wn, *Ln, *Ltn;    // W* between a step's stages (avg keeps W^n), and the stage-1 L and
-                            // L_t (rows of the layer depths only), FP64
+  double *Wn, *Ln, *Ltn;    // W* between a step's stages (avg keeps W^n), and the layer depths'
+                            // stage-1 L and L_t ([layer][cell], lower first), FP64
   void *incR;               // [4][cell] stage-1 part of the stage-2 momentum increment, type R
   void *srec;               // side records [tile][layer][vector][32][16 bytes], type R (lower layer first)
   void *omg;                // omega_H / gamma_H of eta1 [0] and h2 [1], type R
@@ -91,7 +91,7 @@ struct Dev {
   unsigned char *pos_flag;  // [2][cs]
   void *pos_hbar;           // [2][cs], type R
                             // (written by one reconstruction for the next)
-  float *wdev;              // [6][cell] max_k |omega_k / gamma_k - 1| (harvesting)
+  float *wdev;              // [6][cell] max_k |omega_k / gamma_k - 1| (harvesting; scratch)
   // per edge
   // (one aligned vector for what a thread takes at once: an edge's results
   // were read by the update as 78 single values per cell, now as 30 vectors:
@@ -103,8 +103,8 @@ struct Dev {
   void *hrefe;              // [2][edge] R1 - B at the Gauss points, type R
   void *hc;                 // [2][edge] edge-centre blended level deviations, type R
   double *ept;              // [edge][layer][point][side][4] double form: the sides' level deviation, velocity
-                            // along n and t, inverse root of the depth, from k_iface for k_edge
-  int *wl;                  // [2 * edge] (edge << 1 | layer) units left to the deferred edge pass
+                            // along n and t, inverse root of the depth, from k_iface for k_edge (scratch)
+  int *wl;                  // [2 * edge] (edge << 1 | layer) units left to the deferred edge pass (scratch)
   int *wl_count;            // their number (zeroed before each fused edge launch)
   // Gauss-point sums (weights 1/2), deviations, by layer (0 lower), type R but for eM
   void *eF;                 // [layer][edge][4] F (2), F_t (2) of the discharge
@@ -1338,7 +1338,7 @@ __device__ __forceinline__ double update_unit(const Dev &d, const Par &p, int j,
     // in R (their residuals are R), each added to the FP64 state once
     double nw[3], was[3];
     double *now = (stage == 1 ? d.Wn : d.avg) + (size_t)v0 * N + j;
-    double *Ln = d.Ln + (size_t)v0 * N + j, *Ltn = d.Ltn + (size_t)v0 * N + j;
+    double *Ln = d.Ln + (size_t)l * N + j, *Ltn = d.Ltn + (size_t)l * N + j;
     R *inc = (R *)d.incR + (size_t)(l == 1 ? 0 : 2) * N + j;
     for (int k = 0; k < 3; k++) was[k] = d.avg[(size_t)(v0 + k) * N + j];
     if (stage == 1) {
