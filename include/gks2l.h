@@ -314,6 +314,9 @@ int gks2l_mlp_forward(const float *d_X, int32_t n, const float *d_params, float 
 #define GKS2L_GATE_KERNELS 4
 #define GKS2L_GATE_VARIANTS 16
 int gks2l_set_launch_shapes(gks2l_ctx *ctx, const int32_t shapes[4]);
+/* The interface, edge and update kernels' shapes alone: the gate's variant
+ * stays as it is, also where none has been chosen. */
+int gks2l_set_kernel_shapes(gks2l_ctx *ctx, const int32_t shapes[3]);
 
 /* Autotuner: advances the state by GKS2L_LAUNCH_SHAPES * n_steps full steps,
  * exactly as gks2l_advance would, timing the interface, edge and update
@@ -321,7 +324,9 @@ int gks2l_set_launch_shapes(gks2l_ctx *ctx, const int32_t shapes[4]);
  * for each. With the gate on it then times GKS2L_GATE_VARIANTS * (n_steps + 1)
  * more steps, whole steps per gate variant (the gate overlaps other kernels,
  * so its own time does not decide), and keeps the fastest. Writes the
- * choices to shapes[4]. Requires a state and phase at a step boundary;
+ * choices to shapes[4]; with the gate off shapes[3] is the variant last chosen,
+ * 0 where none has been (passing that 0 to gks2l_set_launch_shapes chooses
+ * variant 0; gks2l_set_kernel_shapes takes the other three). Requires a state and phase at a step boundary;
  * returns the run's status like gks2l_advance with t_out. */
 int gks2l_autotune(gks2l_ctx *ctx, int32_t n_steps, int32_t shapes[4]);
 

@@ -1986,14 +1986,22 @@ int gks2l_profile_kernels(gks2l_ctx *c, int32_t n_steps, double ms[6]) {
   return GKS2L_OK;
 }
 
-int gks2l_set_launch_shapes(gks2l_ctx *c, const int32_t shapes[4]) {
+int gks2l_set_kernel_shapes(gks2l_ctx *c, const int32_t shapes[3]) {
   if (!c || !shapes) return GKS2L_EINVAL;
   for (int k = 0; k < 3; k++)
     if (shapes[k] < 0 || shapes[k] >= kShapes) return GKS2L_EINVAL;
-  if (shapes[3] < 0 || shapes[3] >= kGateVariants) return GKS2L_EINVAL;
-  for (int k = 0; k < 4; k++) c->shape[k] = shapes[k];
-  c->gate_auto = false;
+  for (int k = 0; k < 3; k++) c->shape[k] = shapes[k];
   drop_graph(c);
+  return GKS2L_OK;
+}
+
+int gks2l_set_launch_shapes(gks2l_ctx *c, const int32_t shapes[4]) {
+  if (!c || !shapes) return GKS2L_EINVAL;
+  if (shapes[3] < 0 || shapes[3] >= kGateVariants) return GKS2L_EINVAL;
+  const int rc = gks2l_set_kernel_shapes(c, shapes);
+  if (rc) return rc;
+  c->shape[3] = shapes[3];
+  c->gate_auto = false;
   return GKS2L_OK;
 }
 

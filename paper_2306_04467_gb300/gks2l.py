@@ -79,6 +79,7 @@ SIGNATURES = {
     "gks2l_stats": (_I, [_P, ctypes.POINTER(gks2l_stats_t)]),
     "gks2l_profile_kernels": (_I, [_P, ctypes.c_int32, ctypes.POINTER(ctypes.c_double * 6)]),
     "gks2l_set_launch_shapes": (_I, [_P, ctypes.POINTER(ctypes.c_int32 * 4)]),
+    "gks2l_set_kernel_shapes": (_I, [_P, ctypes.POINTER(ctypes.c_int32 * 3)]),
     "gks2l_autotune": (_I, [_P, ctypes.c_int32, ctypes.POINTER(ctypes.c_int32 * 4)]),
     "gks2l_alu_peaks": (_I, [_P, ctypes.POINTER(ctypes.c_double * 2)]),
     "gks2l_set_mlp": (_I, [_P, _P, ctypes.c_size_t]),
@@ -172,7 +173,6 @@ class Solver:
             rc = L.gks2l_create_ensemble(len(meshes), arr, ctypes.byref(params), ctypes.byref(h))
         _check(rc, "gks2l_create")
         self._h = h
-        self._gate_variant = 0
         nbytes = ctypes.c_size_t(0)
         _check(L.gks2l_workspace_bytes(h, ctypes.byref(nbytes)), "gks2l_workspace_bytes")
         self.device = torch.device(device)
@@ -272,22 +272,24 @@ class Solver:
     def set_launch_shapes(self, shapes):
         """Launch shapes (0..4) of the interface, edge and update kernels and,
         as a fourth entry, the gate variant (0..15: kernel = v % 4, placement
-        = v // 4 % 2, edge path = v // 8; kept at the current choice when
-        only three are given)."""
+        = v // 4 % 2, edge path = v // 8). With three entries the gate's
+        variant stays as it is, chosen or not."""
         shapes = [int(x) for x in shapes]
         if len(shapes) == 3:
-            shapes.append(self._gate_variant)
-        b = (ctypes.c_int32 * 4)(*shapes)
-        _check(load().gks2l_set_launch_shapes(self._h, ctypes.byref(b)), "gks2l_set_launch_shapes")
-        self._gate_variant = shapes[3]
+            b = (ctypes.c_int32 * 3)(*shapes)
+            _check(load().gks2l_set_kernel_shapes(self._h, ctypes.byref(b)), "gks2l_set_kernel_shapes")
+        else:
+            b = (ctypes.c_int32 * 4)(*shapes)
+            _check(load().gks2l_set_launch_shapes(self._h, ctypes.byref(b)), "gks2l_set_launch_shapes")
 
     def autotune(self, n_steps=2):
         """Time each launch shape for n_steps steps (they advance the state);
         keep the fastest per kernel (and, with the gate on, the faster gate
-        kernel by whole steps) and return the four choices."""
+        kernel by whole steps) and return the four choices (the gate off: the
+        last is the variant last chosen, 0 for none; pass the first three to
+        set_launch_shapes to leave it open)."""
         b = (ctypes.c_int32 * 4)()
         _check(load().gks2l_autotune(self._h, int(n_steps), ctypes.byref(b)), "gks2l_autotune")
-        self._gate_variant = b[3]
         return list(b)
 
     def alu_peaks(self):
