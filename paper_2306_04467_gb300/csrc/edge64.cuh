@@ -1,5 +1,5 @@
 // The double form's interface levels and edge solution (the single form's are
-// iface_unit and edge_unit in stage.cuh; edge_unit<double> comes here).
+// iface_unit and edge_unit in stage.cuh).
 //
 // On this GPU the FP64 pipe has two lanes per SM, so every kernel of the
 // double form runs at 89-92% of it and its time is its count of FP64

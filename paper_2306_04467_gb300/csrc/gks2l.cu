@@ -523,10 +523,10 @@ __global__ void k_harvest(Dev d, const int *perm, float tol, const float *logit_
 
 // the edge unit of a form
 template <typename R, bool FUSED = false, bool PAIRED = false, bool POS = false, bool HAVE = false>
-__device__ __forceinline__ bool edge_any(const Dev &d, const Par &p, int e, int ell, int q, int stage, R out[12],
+__device__ __forceinline__ bool edge_any(const Dev &d, const Par &p, int e, int ell, int q, R out[12],
                                          R *blend = nullptr, R *own = nullptr) {
   if constexpr (sizeof(R) == 8) return edge_unit64<FUSED, PAIRED, POS, HAVE>(d, p, e, ell, q, out, blend, own);
-  else return edge_unit<R, FUSED, PAIRED, POS>(d, p, e, ell, q, stage, out, blend, own);
+  else return edge_unit<R, FUSED, PAIRED, POS>(d, p, e, ell, q, out, blend, own);
 }
 
 // The edge's results from its two points: the q = 0 thread takes the mean of
@@ -603,7 +603,7 @@ __device__ __forceinline__ void edge_body(const Dev &d, const Par &p, int stage)
   // its instance's dt is known, so the unit's loads issue at once; only
   // edges of instances still running are written
   R out[12], own[2];
-  edge_any<R, false, true, POS, true>(d, p, ee, ell, q, stage, out, nullptr, own);
+  edge_any<R, false, true, POS, true>(d, p, ee, ell, q, out, nullptr, own);
   const bool ok = e < d.ne && running(d, d.eg[4 * (size_t)ee + 3]);
   own_write<R>(d, e, ell, q, own, ok);
   R avg[6];
@@ -624,7 +624,7 @@ __device__ __forceinline__ void edge_fused_body(const Dev &d, const Par &p, int 
   int e = tid >> 2, ell = (tid >> 1) & 1, q = tid & 1;
   const int ee = e < d.ne ? e : d.ne - 1;
   R out[12], bl = 0, own[2];
-  const bool done = edge_any<R, true, true>(d, p, ee, ell, q, stage, out, &bl, own);
+  const bool done = edge_any<R, true, true>(d, p, ee, ell, q, out, &bl, own);
   if (!done) {
     for (int k = 0; k < 12; k++) out[k] = 0;
   }
@@ -668,7 +668,7 @@ __global__ void __launch_bounds__(128) k_edge_deferred(Dev d, Par p, int stage) 
     const int item = d.wl[i < n ? i : n - 1];
     const int e = item >> 1, ell = item & 1;
     R out[12];
-    edge_any<R>(d, p, e, ell, q, stage, out);
+    edge_any<R>(d, p, e, ell, q, out);
     R avg[6];
     edge_mean<R>(d, e, q, out, avg);
     if (i >= n) continue;

@@ -147,8 +147,8 @@ template <typename R> __host__ __device__ __forceinline__ R pv(double d, float f
 template <> __host__ __device__ __forceinline__ double pv<double>(double d, float) { return d; }
 template <> __host__ __device__ __forceinline__ float pv<float>(double, float f) { return f; }
 
-// erf(x) given ex = e^{-x^2}, which the caller has formed already: in FP64
-// the library erf; in FP32 the rational approximation 7.1.26 of Abramowitz
+// erf(x) of the single form given ex = e^{-x^2}, which the caller has formed
+// already (the double form's is half_erf): the rational approximation 7.1.26 of Abramowitz
 // and Stegun (Handbook of Mathematical Functions, after Hastings),
 // erf(|x|) = 1 - P(t) e^{-x^2}, P(t) = a1 t + ... + a5 t^5, t = 1/(1 + p|x|),
 // absolute error at most 1.5e-7, with P re-expanded about t = 1 in
@@ -160,7 +160,6 @@ template <> __host__ __device__ __forceinline__ float pv<float>(double, float f)
 // velocities of a state near rest keep their size in the half-space moments'
 // erf terms, which enter the deviation h-bar - h_b directly.
 template <typename R> __host__ __device__ __forceinline__ R erf_ex(R x, R ex);
-template <> __host__ __device__ __forceinline__ double erf_ex<double>(double x, double) { return erf(x); }
 template <> __host__ __device__ __forceinline__ float erf_ex<float>(float x, float ex) {
   const float ax = x < 0.f ? -x : x;
   const float t = 1.f / (1.f + 0.3275911f * ax);
@@ -173,9 +172,6 @@ template <> __host__ __device__ __forceinline__ float erf_ex<float>(float x, flo
   const float e = (1.f - ex) - ex * s * q;
   return x < 0.f ? -e : e;
 }
-template <typename R> __host__ __device__ __forceinline__ R r_erfc(R x);
-template <> __host__ __device__ __forceinline__ double r_erfc<double>(double x) { return erfc(x); }
-template <> __host__ __device__ __forceinline__ float r_erfc<float>(float x) { return erfcf(x); }
 template <typename R> __host__ __device__ __forceinline__ R r_exp(R x);
 template <> __host__ __device__ __forceinline__ double r_exp<double>(double x) { return exp(x); }
 // single precision on the device: the hardware exponential (a few ulp; the
@@ -661,13 +657,11 @@ template <> struct Rn<double> {
   static __device__ __forceinline__ double add(double a, double b) { return __dadd_rn(a, b); }
   static __device__ __forceinline__ double sub(double a, double b) { return __dsub_rn(a, b); }
   static __device__ __forceinline__ double fma(double a, double b, double c) { return __fma_rn(a, b, c); }
-  static __device__ __forceinline__ double rcp(double a) { return __drcp_rn(a); }
 #else
   static double mul(double a, double b) { return a * b; }
   static double add(double a, double b) { return a + b; }
   static double sub(double a, double b) { return a - b; }
   static double fma(double a, double b, double c) { return std::fma(a, b, c); }
-  static double rcp(double a) { return 1.0 / a; }
 #endif
 };
 
@@ -903,7 +897,7 @@ __host__ __device__ __forceinline__ void time_ints2(R tau, R delta, R qd[5], R q
   time_ints_e<R>(tau, delta, eh * eh, emh * (1 + eh), qd);
 }
 
-// One layer at one Gauss point, local frame (x along the normal from L to R).
+// One layer at one Gauss point in the single form, local frame (x along the normal from L to R).
 // Depths h_l = href + dl, h_r = href + dr. Returns the value and time
 // derivative at the stage start of the flux F and of the interface variables
 // W (fit of the two time integrals over delta and delta/2), as deviations:
@@ -912,6 +906,7 @@ template <typename R>
 __host__ __device__ inline void gks_layer(R href, R dl, R dr, R Ul, R Vl, R Ur, R Vr, const R dnl[3],
                                           const R dtl[3], const R Dl[2], const R dnr[3], const R dtr[3],
                                           const R Dr[2], R g, R tau, R delta, R F[3], R Ft[3], R W[3], R Wt[3]) {
+  static_assert(sizeof(R) == 4, "the double form's is gks_layer64");
   const R hlR = href + dl, hrR = href + dr;
   const R dlr = dl - dr;                          // h_l - h_r, exact at rest
   const R laml = 1 / (g * hlR), lamr = 1 / (g * hrR);
@@ -1007,22 +1002,23 @@ __host__ __device__ inline void gks_layer(R href, R dl, R dr, R Ul, R Vl, R Ur, 
   for (int k = 0; k < 3; k++) { Wt[k] = wt[k]; Ft[k] = ft[k]; }
 }
 
-// Blended level deviation at one point (Sec. 2.3): d^r + xi (d^l - d^r) with
+// Blended level deviation at one point in the single form (Sec. 2.3): d^r + xi (d^l - d^r) with
 // xi = erfc((U_n^l + U_n^r)/2)/2, U_n = (m . n) / h on each side. Written
 // with explicitly rounded operations so that the interface kernel and the
 // fused edge kernel, which both form it, get the same value whatever the
 // compiler does with the code around it.
 template <typename R>
 __host__ __device__ __forceinline__ R blend_level(R dl, R hl, R mxl, R myl, R dr, R hr, R mxr, R myr, R n0, R n1) {
+  static_assert(sizeof(R) == 4, "the double form's is blend64");
   using O = Rn<R>;
   const R ul = O::mul(O::fma(mxl, n0, O::mul(myl, n1)), O::rcp(hl));
   const R ur = O::mul(O::fma(mxr, n0, O::mul(myr, n1)), O::rcp(hr));
-  const R xi = O::mul((R)0.5, r_erfc<R>(O::mul((R)0.5, O::add(ul, ur))));
+  const R xi = O::mul((R)0.5, erfcf(O::mul((R)0.5, O::add(ul, ur))));
   return O::fma(xi, O::sub(dl, dr), dr);
 }
 
 // ---------------------------------------------------- interface (iface) unit
-// Blended level deviation of layer ell at edge e (Sec. 2.3), the mean over
+// Blended level deviation of layer ell at edge e in the single form (Sec. 2.3), the mean over
 // the two Gauss points of h-hat = xi h^l + (1 - xi) h^r with
 // xi = erfc((U_n^l + U_n^r)/2)/2; the lower layer is blended as the water
 // level eta1 (B is continuous). Each side's record is loaded once for both
@@ -1030,6 +1026,7 @@ __host__ __device__ __forceinline__ R blend_level(R dl, R hl, R mxl, R myl, R dr
 // 121 us at 1.04 M triangles; the double form takes them.)
 template <typename R>
 __host__ __device__ __forceinline__ R iface_unit(const Dev &d, int e, int ell) {
+  static_assert(sizeof(R) == 4, "the double form's is iface_unit64");
   const EdgeIds g = edge_ids(d, e);
   R x[2][4], n[2], vl[2][3], vr[2][3];
   for (int q = 0; q < 2; q++) load_n<R, 4>((const R *)d.exi + ((size_t)q * d.ne + e) * 4, x[q]);
@@ -1071,7 +1068,7 @@ __host__ __device__ __forceinline__ void plane_grad(const Dev &d, int c, int whi
 }
 
 // ------------------------------------------------------------- edge unit
-// Interface solution of layer ell at Gauss point q of edge e, global frame:
+// Interface solution of the single form, layer ell at Gauss point q of edge e, global frame:
 // out[0..2] = F, out[3..5] = F_t, out[6..8] = W, out[9..11] = W_t (deviations).
 // Returns true when out was computed.
 // FUSED (runs with the troubled-cell gate, where most cells take the linear
@@ -1090,8 +1087,9 @@ __host__ __device__ __forceinline__ void plane_grad(const Dev &d, int c, int whi
 // layer has point depths below half its average, the side velocity is
 // bounded by the edge's two cells' average velocities of the layer.
 template <typename R, bool FUSED = false, bool PAIRED = false, bool POS = false>
-__host__ __device__ inline bool edge_unit(const Dev &d, const Par &p, int e, int ell, int q, int stage, R out[12],
+__host__ __device__ inline bool edge_unit(const Dev &d, const Par &p, int e, int ell, int q, R out[12],
                                           R *blend = nullptr, R *own = nullptr) {
+  static_assert(sizeof(R) == 4, "the double form's is edge_unit64");
   const EdgeIds g = edge_ids(d, e);
   const int cL = g.L, cR = g.R, xf = g.xf;
   R x[4], n[2];
@@ -1102,7 +1100,6 @@ __host__ __device__ inline bool edge_unit(const Dev &d, const Par &p, int e, int
   // time integrals over dt and dt/2 (the S2O4 construction repeated from the
   // intermediate state, reading R20)
   const R delta = dt;
-  (void)stage;
   const R href = ref_depth<R>(d, ell, e, q);
   SideVals<R> s[2];
 #ifdef __CUDA_ARCH__
