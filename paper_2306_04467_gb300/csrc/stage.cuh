@@ -54,11 +54,8 @@ constexpr int NCOEF = 10;    // per variable: c0 (value offset) + 9 Taylor coeff
 // (1.04 M triangles; the fused k_edgef, bound by issue, 287 -> 295 us).
 constexpr int NREC = 36;
 
-// Device view of the workspace. R-typed arrays are stored as void* and cast. A
-// multiple of 16 bytes, so that the kernels' next argument, Par, starts on 16 bytes
-// and its constants come by vector loads: at 8 bytes off k_edge<float> spills two of
-// its 96 registers, 291 us in place of 283 (1.04 M triangles).
-struct alignas(16) Dev {
+// Device view of the workspace. R-typed arrays are stored as void* and cast.
+struct Dev {
   int nt, ne, ninst;
   int cs;                   // stride of per-cell arrays (nt rounded up to 32)
   // per cell
@@ -80,8 +77,8 @@ struct alignas(16) Dev {
   double *avg;              // state averages [v][cell] (FP64)
   void *dq, *dg;            // deviation mirrors [pair][cell][2] and gradients [pair][cell][2][2], type R
   void *hrefc;              // R1 - B_j per cell, type R
-  double *Wn, *Ln, *Ltn;    // W* between a step's stages (avg keeps W^n), and the layer depths'
-                            // stage-1 L and L_t ([layer][cell], lower first), FP64
+  double *Wn, *Ln, *Ltn;    // W* between a step's stages (avg keeps W^n), and the stage-1 L and
+                            // L_t (rows of the layer depths only, 0 and 3), FP64
   void *incR;               // [4][cell] stage-1 part of the stage-2 momentum increment, type R
   void *srec;               // side records [tile][layer][vector][32][16 bytes], type R (lower layer first)
   void *omg;                // omega_H / gamma_H of eta1 [0] and h2 [1], type R
@@ -101,7 +98,7 @@ struct alignas(16) Dev {
   // k_update<float> 38 -> 31 us at 181 k triangles, 158 -> 152 at 1.04 M)
   const int *eg;            // [edge][4] L cell, R cell, the R side's transform, instance
   const void *en;           // [edge][2] unit normal from L to R, type R
-  const double *eb0, *eb1;  // B at the two Gauss points
+  const double *eb;         // [point][edge] B at the Gauss points
   const void *exi;          // [point][edge][4] Gauss point in the L and the R side's scaled frame, type R
   void *hrefe;              // [2][edge] R1 - B at the Gauss points, type R
   void *hc;                 // [2][edge] edge-centre blended level deviations, type R
@@ -128,6 +125,11 @@ struct alignas(16) Dev {
   unsigned long long *gate_count;
   const double *xf;         // [code*4] 2x2 linear parts of image transforms
 };
+// The kernels' next argument, Par, starts on 16 bytes, and its constants come by
+// vector loads: at 8 bytes off k_edge<float> spills two of its 96 registers, 291 us in
+// place of 283 (1.04 M triangles). Not by alignas, which has the compiler load the
+// pointers themselves in pairs too: k_update<float> 886 us in place of 866 (8 M).
+static_assert(sizeof(Dev) % 16 == 0, "an even number of pointers");
 
 struct Par {
   double g, chi, cfl, eps, eps_num, gam_hi, weno_eps;
@@ -1338,7 +1340,7 @@ __device__ __forceinline__ double update_unit(const Dev &d, const Par &p, int j,
     // in R (their residuals are R), each added to the FP64 state once
     double nw[3], was[3];
     double *now = (stage == 1 ? d.Wn : d.avg) + (size_t)v0 * N + j;
-    double *Ln = d.Ln + (size_t)l * N + j, *Ltn = d.Ltn + (size_t)l * N + j;
+    double *Ln = d.Ln + (size_t)v0 * N + j, *Ltn = d.Ltn + (size_t)v0 * N + j;
     R *inc = (R *)d.incR + (size_t)(l == 1 ? 0 : 2) * N + j;
     for (int k = 0; k < 3; k++) was[k] = d.avg[(size_t)(v0 + k) * N + j];
     if (stage == 1) {
