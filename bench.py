@@ -118,13 +118,12 @@ WORK_PER_UNIT = {
 }
 # FP32 flops per unit that the hardware executes (ncu sm__sass_thread_inst_
 # executed_op_f{add,mul,fma} with FMA = 2): reported beside the algorithmic
-# counts as the overhead ratio. recon, gate, edge_fused, update: one step of
-# the large configuration at 1416 x 177 squares (501,264 triangles); iface and
-# edge (the plain form's): the lake at 512 x 512 squares, captured before the
-# edge kernels' last instruction cuts. The FP32 arithmetic has not changed
-# since these captures; its loads, stores and launches have.
-EXECUTED_FP32_PER_UNIT = {"recon": 2214, "gate": 258, "iface": 836, "edge": 5405, "edge_fused": 5500,
-                          "update": 319}
+# counts as the overhead ratio. One step of the large configuration at 1416 x
+# 177 squares (501,264 triangles), the current kernels, both stages' mean: iface
+# and edge in the plain form, the others with the gate (recon with the gate's own
+# kernel beside it, recon_gate with the decisions inside).
+EXECUTED_FP32_PER_UNIT = {"recon": 2209, "recon_gate": 2467, "gate": 266, "iface": 873, "edge": 5257,
+                          "edge_fused": 5497, "update": 321}
 # Measured FMA-chain peaks of a GB300 (TFLOP/s, 2 flops per FMA); the
 # bench replaces them with the same run's own measurement.
 PEAK_TFLOPS = {"fp32": 76.5, "fp64": 1.254}
@@ -133,7 +132,7 @@ PEAK_TFLOPS = {"fp32": 76.5, "fp64": 1.254}
 # current kernels on the large configuration at 1416 x 177 squares (inputs
 # larger than L2); the bench scales them to its launch by the units. A kernel
 # is listed only while it is unchanged since that capture.
-TRAFFIC_PER_UNIT = {"recon": 1017.0, "edge_fused": 362.7, "update": 486.0}
+TRAFFIC_PER_UNIT = {"recon": 1033.6, "edge_fused": 363.4, "update": 480.2}
 
 
 KERNEL_NAME = {"edge_fused": "k_edgef", "edge_deferred": "k_edge_deferred"}
@@ -641,7 +640,8 @@ def main():
     roof["algorithmic_bytes_per_unit"] = by_unit
     roof["units_per_launch"] = units
     roof["launch_ms"] = top_ms
-    ex = EXECUTED_FP32_PER_UNIT.get(top)
+    inside = rh["shapes"][3] in (4, 12)    # the reconstruction takes the gate's decisions
+    ex = EXECUTED_FP32_PER_UNIT.get("recon_gate" if top == "recon" and inside else top)
     roof["executed_fp32_per_unit"] = ex
     roof["overhead_executed_over_algorithmic"] = (ex / fl_unit) if ex else None
     roof["per_kernel"] = hf["roofline_frac"]
@@ -649,8 +649,8 @@ def main():
     ksum = sum(kern[x] for x in timed)
     share = {x: kern[x] / ksum for x in timed}
     # step start, then per stage reconstruction, two edge kernels, update and,
-    # unless the reconstruction takes its decisions (variants 4 and 12), the gate
-    launches_per_step = 1 + 2 * (4 if rh["shapes"][3] in (4, 12) else 5)
+    # unless the reconstruction takes its decisions, the gate
+    launches_per_step = 1 + 2 * (4 if inside else 5)
 
     def strip(w):
         return {"workload": w["workload"], "n_tri": w["n_tri"],

@@ -234,9 +234,10 @@ int gks2l_stats(gks2l_ctx *ctx, gks2l_stats_t *out);
  * A 24 -> 32 -> 32 -> 1 MLP (ReLU hidden layers, sigmoid output) predicts per
  * cell whether the nonlinear WENO weights of the reconstruction would depart
  * from the linear ones; cells it calls smooth take the linear P3
- * reconstruction and a blending weight w = 1. The network runs on a second
- * stream beside each stage's reconstruction or edge kernels, on the state
- * that stage reconstructed, and its decisions apply to the next
+ * reconstruction and a blending weight w = 1. The network runs on the state
+ * that a stage reconstructs, inside the reconstruction (the single form, while
+ * no variant or variant 4 or 12 is chosen) or on a second stream beside the
+ * reconstruction or the edge kernels, and its decisions apply to the next
  * reconstruction; gks2l_set_state runs it once on the state it sets, for
  * the first stage (the first stage after gks2l_set_mlp is the plain
  * method). gks2l_set_mlp creates that stream. Parameters are a float vector
@@ -262,8 +263,8 @@ int gks2l_set_mlp(gks2l_ctx *ctx, const float *params, size_t n_floats);
  * sqrt(sum of their squares + weno_eps |Omega| (1 + q0^2)). d_logits: null,
  * or n_tri floats for the logits the fused gate computes for these cells
  * (needs a network loaded by gks2l_set_mlp). All pointers are device memory.
- * Synchronises the stream; the state is not changed (a gate loaded with
- * gks2l_set_mlp takes its decisions for the next stage from this state). */
+ * Synchronises the stream; the state and the gate's decisions for the next
+ * stage are not changed. */
 int gks2l_harvest(gks2l_ctx *ctx, float tol, float *d_features, float *d_labels, float *d_logits);
 
 /* Gradient of the weighted logistic loss
@@ -271,8 +272,10 @@ int gks2l_harvest(gks2l_ctx *ctx, float tol, float *d_features, float *d_labels,
  * of n samples (device d_X[n][24], d_y[n] in {0, 1}) for parameters d_params
  * (device, GKS2L_MLP_NPARAM floats): writes d_grads[GKS2L_MLP_NTRAIN] (sums
  * over the samples) and d_loss[1]. BF16 tensor cores, FP32 sums in a fixed
- * order (the result is reproducible). Takes stream-ordered scratch of about
- * 7.6 KB per 64 samples (at most 18 MB). */
+ * order (the result is reproducible). Takes stream-ordered scratch of 7.6 KB
+ * per block of 64 samples, of which there are at most two per SM (2.3 MB on
+ * 152 SMs; with more samples a block takes several times 64), from the device's
+ * default pool: a call after a synchronisation maps it anew, some 170 us. */
 int gks2l_mlp_grad(const float *d_X, const float *d_y, int32_t n, const float *d_params, float pos_weight,
                    float *d_grads, float *d_loss, void *stream);
 

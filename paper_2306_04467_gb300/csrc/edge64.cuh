@@ -5,7 +5,7 @@
 // double form runs at 89-92% of it and its time is its count of FP64
 // operations (library calls in pipe slots: exp 15, erf 45, erfc 62, expm1 19,
 // a/b 8, sqrt 8, 1/x 5, rsqrt 5). The formulation here is the one with the
-// fewest (measured with 501 k triangles, 752 k edges): 1211 -> 777 per edge,
+// fewest (measured with 501 k triangles, 753 k edges): 1211 -> 777 per edge,
 // layer and point (k_edge<double> 6595 -> 4274 us) and 341 -> 274 per edge and
 // layer (k_iface<double> 954 -> 763 us), then, with the sides' values kept by
 // k_iface and the results rotated once per edge, 633 (k_edge<double> 582 -> 496
@@ -28,7 +28,8 @@ using D64 = Rn<double>;
 
 // erf(z)/2 for |z| <= 1/2 by the Maclaurin series 1/sqrt(pi) sum_n (-1)^n
 // z^(2n+1) / (n! (2n+1)); the first term left out is below 2^-58 of the sum.
-// Larger arguments (Froude numbers above 0.7) take the library's.
+// Larger arguments take the library's: normal Froude numbers above 0.5 (z = U /
+// sqrt(G h)), and in the blend U_n^l + U_n^r above 1 (z is half their sum).
 constexpr int kErfTerms = 13;
 struct ErfSeries {
   double c[kErfTerms];

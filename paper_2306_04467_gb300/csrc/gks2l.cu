@@ -11,8 +11,8 @@
 //   k_update  (cell)                 fluxes, sources, S2O4 update, Gauss-theorem
 //                                    gradients (Eqs. SWE-semi-flux, slope-1, S2O3),
 //                                    CFL reduction
-// With the learned troubled-cell gate, k_gate (next stage's mask) runs on a
-// second stream, and k_iface + k_edge become k_edgef (both in one pass where
+// With the learned troubled-cell gate, k_recon (single form) or k_gate on a
+// second stream decides the next stage's mask, and k_iface + k_edge become k_edgef (both in one pass where
 // the plane gradients carry no weight) + k_edge_deferred (the other edges).
 // A step is k_step_begin + two stages, captured once into a CUDA graph.
 #include <cuda_runtime.h>
@@ -329,15 +329,16 @@ __global__ void __launch_bounds__(TW * 6 / ReconCfg<R>::VP, ReconCfg<R>::BLOCKS)
   }
 }
 
-// Troubled-cell gate (not part of the paper). It runs on a second stream
-// beside the interface and edge kernels of a stage, on the state that stage
+// Troubled-cell gate (not part of the paper) where the reconstruction does not
+// take its decisions along. It runs on a second stream beside the interface and edge kernels of a stage, on the state that stage
 // reconstructed, and leaves for the next reconstruction the mask of cells it
 // calls smooth. Persistent warps keep the network in registers and walk over
 // tiles of 32 cells: the 24 features of each cell go to a shared-memory tile,
 // the network runs on the tensor cores, and the warp writes the tile's mask
 // (cells past the end or of finished instances count as smooth).
-// k_gate: as many as its registers allow, latency-bound warps (alone 26.5 ->
-// 18.0 us at 181 k triangles against two per SM)
+// k_gate: latency-bound warps. FP32: 96 registers, five blocks fit (alone 26.5 ->
+// 18.0 us at 181 k triangles against two per SM); FP64: 164, three fit (76 us with
+// two, 70 with three, 71 with five, the gated stage the same with all)
 constexpr int GATE_BLOCKS_PER_SM = 5;
 constexpr int GATE_TC_BLOCKS_PER_SM = 2;   // k_gate_tc, times the variant's factor
 

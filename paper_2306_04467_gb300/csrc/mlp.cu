@@ -85,7 +85,9 @@ __device__ __forceinline__ bool aligned16(const float *p) { return (reinterpret_
 // memory, rows, six small products, sums; so rows come as 16-byte vectors
 // requested before the network is packed, and the warps' sums meet in shared
 // memory, which leaves the reduction a quarter of the partials. A training
-// step (gradient, reduction, Adam) of 8192 samples: 32.1 -> 23.9 us.
+// step (gradient, reduction, Adam) of 8192 samples, steps queued: 32.1 -> 23.9 us,
+// 21.4 with the reduction's launch chained; alone after a synchronisation 206 -> 195,
+// most of it the partials' memory, which the default pool has given back.
 constexpr int NPART = MLP_NTRAIN + 1;
 
 __global__ void __launch_bounds__(TPB) k_mlp_grad(const float *X, const float *y, int n, const float *P, float pos_w,
